@@ -183,10 +183,8 @@ __device__ __forceinline__ void run_item(const PscBatchBox& b, int pass, int til
   const Tctx strided{tid % W, tid / W, tile % gx, tile / gx, W, LPL, gx, smem};
   switch (pass) {
     case BP_FAMP:
-      if (tid == 0) {
-        if (STAGE == 1 && b.cfl_on) ctrl->umax_bits = 0ull;
-        b_famp<float>(a.d, a.in, ctrl, b.kF2, b.eps_inj, b.forcing, STAGE == 1 ? 1 : 0);
-      }
+      if (tid == 0 && STAGE == 1 && b.cfl_on) ctrl->umax_bits = 0ull;
+      if (tid < 32) b_famp<float>(a.d, a.in, ctrl, b.kF2, b.eps_inj, b.forcing, STAGE == 1 ? 1 : 0, tid);
       break;
     case BP_ZINV: b_zinv<float, N, false, W>(a, strided); break;
     case BP_YINV: b_yinv<float, N, YMODE_RHS, W>(a, strided); break;
@@ -227,7 +225,7 @@ __device__ __forceinline__ void run_item(const PscBatchBox& b, int pass, int til
       break;
     }
     default:
-      if (tid == 0) b_hold<float>(a.d, b.U, ctrl, b.kF2);
+      if (tid < 32) b_hold<float>(a.d, b.U, ctrl, b.kF2, tid);
       break;
   }
 }
