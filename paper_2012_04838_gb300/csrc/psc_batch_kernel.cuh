@@ -179,12 +179,17 @@ __device__ __forceinline__ void run_item(const PscBatchBox& b, int pass, int til
   a.phase = nullptr;
   a.shift = 0;
   a.xrow = 0;
+  a.force.on = a.cfl.on = 0;
+  a.share = 1;
   a.st = nullptr;
   const Tctx strided{tid % W, tid / W, tile % gx, tile / gx, W, LPL, gx, smem};
   switch (pass) {
     case BP_FAMP:
-      if (tid == 0 && STAGE == 1 && b.cfl_on) ctrl->umax_bits = 0ull;
-      if (tid < 32) b_famp<float>(a.d, a.in, ctrl, b.kF2, b.eps_inj, b.forcing, STAGE == 1 ? 1 : 0, tid);
+      if (tid < 32)
+        b_famp<float>(a.d, a.in, ctrl,
+                      ForceArgs{1, b.kb, b.kF2_floor, b.forcing, STAGE == 1 ? 1 : 0, STAGE == 1 && b.cfl_on ? 1 : 0,
+                                b.eps_inj},
+                      tid);
       break;
     case BP_ZINV: b_zinv<float, N, false, W>(a, strided); break;
     case BP_YINV: b_yinv<float, N, YMODE_RHS, W>(a, strided); break;
@@ -225,7 +230,7 @@ __device__ __forceinline__ void run_item(const PscBatchBox& b, int pass, int til
       break;
     }
     default:
-      if (tid < 32) b_hold<float>(a.d, b.U, ctrl, b.kF2, tid);
+      if (tid < 32) b_hold<float>(a.d, b.U, ctrl, b.kb, b.kF2_floor, tid);
       break;
   }
 }

@@ -169,6 +169,7 @@ struct psc_sim {
   int wv[SP_N];  // tile-width variant of each strided pass (autotuned at creation)
   int xrow = 0;  // PSC_XPASS_ROWS=1 at creation: the row X pass where the register one exists
   int stall_test = 0;  // PSC_XPASS_STALL_TEST=1 at creation: failure-path test of the TMA waits
+  int share = 1;  // members of the batch being captured (PassArgs::share)
   // launch accounting and optional per-launch event timing
   int64_t launches = 0;
   bool profiling = false;
@@ -483,16 +484,41 @@ PassArgs pass_args(psc_sim* s, const void* in) {
   a.phase = s->ws + s->L.phase;
   a.shift = 0;
   a.xrow = s->xrow;
+  std::memset(&a.force, 0, sizeof(a.force));
+  std::memset(&a.cfl, 0, sizeof(a.cfl));
+  a.share = s->share;
   a.st = s->st;
   return a;
 }
 
-template <typename T>
-void launch_famp(psc_sim* s, const void* in, bool step_start = false) {
-  launch(s, PSC_K_FORCING, 1, [&] {
-    k_famp<T><<<1, 32, 0, s->st>>>(s->d, in, s->ctrl, s->p.kF * s->p.kF, s->p.eps_inj, s->p.forcing,
-                                   step_start ? 1 : 0);
-  });
+// The forcing amplitude of `in`, taken by the z-inverse launch that reads it.
+ForceArgs force_args(const psc_sim* s, bool step_start, bool clear_umax) {
+  const double kF2 = s->p.kF * s->p.kF;
+  ForceArgs f;
+  f.on = 1;
+  f.k2max = kF2 >= 2.0e9 ? 2000000000 : (int)std::floor(kF2);
+  f.kb = 0;
+  while (f.kb < s->d.K && (long long)(f.kb + 1) * (f.kb + 1) <= f.k2max) ++f.kb;
+  f.forcing = s->p.forcing;
+  f.step_start = step_start ? 1 : 0;
+  f.clear_umax = clear_umax ? 1 : 0;
+  f.eps_inj = s->p.eps_inj;
+  return f;
+}
+
+// The CFL time step and its integrating factors, taken by the y-forward launch
+// of stage 1.
+CflArgs cfl_args(const psc_sim* s) {
+  CflArgs c;
+  c.on = 1;
+  c.record_every = s->p.record_every;
+  c.cfl = s->p.cfl;
+  c.dx = 2.0 * M_PI / s->p.N;
+  c.nu = s->p.nu;
+  c.D = s->p.nu / s->p.Sc;
+  c.eu = s->ws + s->L.eu;
+  c.ep = s->ws + s->L.ep;
+  return c;
 }
 
 template <typename T>
@@ -549,8 +575,6 @@ void launch_combine(psc_sim* s, int stage, const CombineArgs& c) {
 // shifted by half a cell (into the z region); the combine averages them.
 template <typename T>
 void rhs_passes(psc_sim* s, const void* in, bool umax, bool step_start = false) {
-  if (umax) cudaMemsetAsync(&s->ctrl->umax_bits, 0, sizeof(unsigned long long), s->st);
-  launch_famp<T>(s, in, step_start);
   // the convective form takes the 8 z-stage streams of the statistics pass and
   // d_y u_z, d_z u_y separately at the y stage
   const bool conv = s->p.nonlinear_form == PSC_NL_CONVECTIVE;
@@ -560,15 +584,11 @@ void rhs_passes(psc_sim* s, const void* in, bool umax, bool step_start = false) 
     a.shift = sh;
     a.want_umax = umax && sh == 0 ? 1 : 0;
     if (nshift == 2 && sh == 0) a.rb = s->ws + s->L.R0;
+    if (sh == 0) a.force = force_args(s, step_start, umax);
+    if (a.want_umax && s->p.cfl > 0.0) a.cfl = cfl_args(s);
     launch(s, PSC_K_ZINV, 1, [&] { s->tb->zinv(a, conv, s->wv[SP_ZINV]); });
     launch(s, PSC_K_YINV, 1, [&] { s->tb->yinv(a, conv ? YMODE_CONVECTIVE : YMODE_RHS, s->wv[SP_YINV]); });
     launch(s, PSC_K_XPASS, 1, [&] { s->tb->xpass(a, conv ? XMODE_CONVECTIVE : XMODE_RHS); });
-    if (a.want_umax && s->p.cfl > 0.0) {
-      launch(s, PSC_K_OTHER, 1, [&] {
-        k_cfl<<<1, 32, 0, s->st>>>(s->ctrl, s->p.cfl, 2.0 * M_PI / s->p.N, s->p.record_every);
-      });
-      launch_iftab<T>(s);
-    }
     launch(s, PSC_K_YFWD, 1, [&] { s->tb->yfwd(a, s->wv[SP_YFWD]); });
     launch(s, PSC_K_ZFWD, 1, [&] { s->tb->zfwd(a, s->wv[SP_ZFWD]); });
   }
@@ -589,7 +609,8 @@ psc_status do_step(psc_sim* s, int nsteps) {
     }
     if (s->p.forcing == PSC_FORCE_HOLD_ENERGY) {
       launch(s, PSC_K_FORCING, 1, [&] {
-        k_hold<T><<<1, 32, 0, s->st>>>(s->d, U, s->ctrl, s->p.kF * s->p.kF);
+        const ForceArgs f = force_args(s, false, false);
+        k_hold<T><<<1, 32, 0, s->st>>>(s->d, U, s->ctrl, f.kb, f.k2max);
       });
     }
     PSC_LAUNCHED("psc_step");
@@ -659,8 +680,7 @@ psc_status do_stats(psc_sim* s, double* Ek, double* Ephi, int cap, int* nshell, 
   const Dims& d = s->d;
   const void* U = s->ws + s->L.U;
   PassArgs a = pass_args(s, U);
-  PSC_CUDA(cudaMemsetAsync(&s->ctrl->umax_bits, 0, sizeof(unsigned long long), s->st));
-  launch_famp<T>(s, U);
+  a.force = force_args(s, false, true);
   launch(s, PSC_K_OTHER, 3, [&] {
     s->tb->zinv(a, true, s->wv[SP_ZINV]);
     s->tb->yinv(a, YMODE_STATS, s->wv[SP_YINV]);
@@ -1034,6 +1054,7 @@ psc_status psc_xpass_probe(int32_t N, int32_t precision, int64_t rows, void* buf
   a.xb = b + L.xb;
   a.tw = b + L.tw;
   a.ctrl = (Ctrl*)(b + L.ctrl);
+  a.share = 1;
   a.st = cs;
   const PassTable* tb = fp64 ? table_f64(N) : table_f32(N);
   for (int i = 0; i < nlaunch; ++i) tb->xpass(a, XMODE_RHS);
@@ -1094,6 +1115,7 @@ psc_status psc_batch_create(psc_sim* const* sims, int32_t n, void* stream, psc_b
     sims[i]->profiling = false;
     step0[i] = sims[i]->step;
     launch0[i] = sims[i]->launches;
+    sims[i]->share = n;
   }
   cudaError_t e = cudaStreamBeginCapture(b->st, cudaStreamCaptureModeRelaxed);
   psc_status st = PSC_OK;
@@ -1112,6 +1134,7 @@ psc_status psc_batch_create(psc_sim* const* sims, int32_t n, void* stream, psc_b
   cudaError_t e2 = cudaStreamEndCapture(b->st, &g);
   for (int i = 0; i < n; ++i) {
     sims[i]->profiling = prof[i];
+    sims[i]->share = 1;
     b->launches_per_step.push_back(sims[i]->launches - launch0[i]);
     sims[i]->step = step0[i];
     sims[i]->launches = launch0[i];
@@ -1172,6 +1195,7 @@ static PscBatchBox box_of(psc_sim* s) {
   const CombineArgs c = combine_args(s, nullptr);
   b.kF2 = c.kF2;
   b.kF2_floor = c.kF2_floor;
+  b.kb = force_args(s, false, false).kb;
   b.eps_inj = s->p.eps_inj;
   b.beta = c.beta;
   b.nu = c.nu;

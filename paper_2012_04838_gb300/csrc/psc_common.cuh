@@ -90,13 +90,27 @@ template <int N> struct PlanD : Plan<N> {
 // Thread and block coordinates of a kernel body: the hardware's in an ordinary
 // launch, or virtual ones when the persistent ensemble kernel runs the body as
 // one item of its work table (then the body must not rely on gridDim beyond gdx).
+// part of parts: which share of a strided pass's transforms the body runs.
 struct Tctx {
   int tx, ty, bx, by, bdx, bdy, gdx;
   unsigned char* smem;  // the body's dynamic shared memory
+  int part = 0, parts = 1;
 };
-__device__ __forceinline__ Tctx hw_ctx(unsigned char* smem) {
-  return Tctx{(int)threadIdx.x, (int)threadIdx.y, (int)blockIdx.x, (int)blockIdx.y,
-              (int)blockDim.x,  (int)blockDim.y,  (int)gridDim.x,  smem};
+// lead: rows of CTAs ahead of the pass's own (PassArgs::force, PassArgs::cfl)
+__device__ __forceinline__ Tctx hw_ctx(unsigned char* smem, int lead = 0) {
+  return Tctx{(int)threadIdx.x, (int)threadIdx.y, (int)blockIdx.x, (int)blockIdx.y - lead,
+              (int)blockDim.x,  (int)blockDim.y,  (int)gridDim.x,  smem, (int)blockIdx.z, (int)gridDim.z};
+}
+// Grids whose strided passes may be cut into shares (Passes::parts): above 256
+// the tiles alone always fill the chip, and the loop bounds stay constants.
+template <int N> constexpr bool kSplit = N <= 256;
+template <int N> __device__ __forceinline__ int share_of(const Tctx& t) { return kSplit<N> ? t.part : 0; }
+// Transforms [t0, t1) of nt that share `part` of `parts` runs (parts <= nt).
+template <int N>
+__device__ __forceinline__ int part_begin(int nt, int part, int parts) {
+  if constexpr (!kSplit<N>) return part * nt;
+  const int per = (nt + parts - 1) / parts;
+  return part * per < nt ? part * per : nt;
 }
 
 // Pointer qualifier of pass inputs: __restrict__ in ordinary launches.  The

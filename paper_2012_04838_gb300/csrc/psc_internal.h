@@ -94,6 +94,22 @@ enum { Z_UX, Z_UY, Z_UZ, Z_DZUY, Z_DZUX, Z_PHI, Z_DZPHI, Z_DZUZ, Z_NSTREAM };
 enum { Y_UX, Y_UY, Y_UZ, Y_WX, Y_DZUX, Y_DYUX, Y_PHI, Y_DYPHI, Y_DZPHI, Y_DYUY, Y_DZUZ, Y_DZUY, Y_NSTREAM };
 constexpr int Y_NSTREAM_ROT = Y_DZUY;  // streams the rotational form and the statistics use
 
+// Scalar work that the first row of CTAs of a launch takes beside the pass
+// (psc_scalars.cuh): the forcing amplitude in the z-inverse of a right-hand
+// side, the CFL time step and integrating factors in the y-forward of stage 1.
+struct ForceArgs {
+  int on;          // 1: the z-inverse launch carries the extra row
+  int kb, k2max;   // the band 0 < |k|^2 <= k2max, |k_i| <= kb
+  int forcing, step_start, clear_umax;
+  double eps_inj;
+};
+struct CflArgs {
+  int on;          // 1: the y-forward launch carries the extra row
+  int record_every;
+  double cfl, dx, nu, D;
+  void *eu, *ep;
+};
+
 struct PassArgs {
   Dims d;
   const void* in;   // stage input, compact 4 fields
@@ -109,6 +125,9 @@ struct PassArgs {
   const void* phase; // exp(i k pi / N), k = -K..K (phase-shift dealiasing)
   int shift;        // 1: evaluate on the grid shifted by half a cell
   int xrow;         // 1: the shared-memory row X pass where the register one exists
+  ForceArgs force;
+  CflArgs cfl;
+  int share;        // boxes whose passes run on the chip at the same time (at least 1)
   cudaStream_t st;
 };
 
@@ -155,7 +174,7 @@ struct PscBatchBox {
   const void* tw;                 // twiddles exp(-2 pi i j / N)
   void* ctrl;                     // the simulation's control block
   double kF2, eps_inj, beta, nu, D, cfl, dx;
-  int kF2_floor, forcing, integrator, scalar_on, record_every, cfl_on;
+  int kb, kF2_floor, forcing, integrator, scalar_on, record_every, cfl_on;
 };
 
 // Grid sizes the persistent kernel runs (FP32-mixed, 2/3 rule, rotational form).

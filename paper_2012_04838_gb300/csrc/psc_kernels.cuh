@@ -1,10 +1,10 @@
 // Pointwise spectral kernels: the stage combine (projection, forcing, scalar
-// source, Lawson IF-RK4 update), forcing amplitude, integrating-factor tables,
-// CFL time step, the FP64 statistics reductions and the initial condition.
+// source, Lawson IF-RK4 update), the deterministic forcing, integrating-factor
+// tables, the FP64 statistics reductions and the initial condition.
 // Kernels that are not templates are static: several units compile this header.
 #pragma once
 
-#include "psc_common.cuh"
+#include "psc_scalars.cuh"
 
 namespace psc {
 
@@ -187,123 +187,14 @@ __global__ void __launch_bounds__(256) k_pressure(Dims d, const void* rb_, void*
   out[i] = mk(kdot.y * ik2 - q.x, -kdot.x * ik2 - q.y);
 }
 
-// Visit the stored modes of the forcing band 0 < |k|^2 <= kF^2, shared out over
-// the 32 lanes of a warp in a fixed order: fn(index, weight).
-template <class F>
-__device__ __forceinline__ void for_band(const Dims& d, double kF2, int lane, const F& fn) {
-  int kb = 0;
-  while ((double)(kb + 1) * (kb + 1) <= kF2 && kb < d.K) ++kb;
-  const int side = 2 * kb + 1, nx = kb + 1;
-  const long long n = (long long)side * side * nx;
-#pragma unroll 4
-  for (long long q = lane; q < n; q += 32) {
-    const int kx = (int)(q % nx);
-    const long long r = q / nx;
-    const int ky = (int)(r % side) - kb, kz = (int)(r / side) - kb;
-    const int k2 = kx * kx + ky * ky + kz * kz;
-    if (k2 == 0 || (double)k2 > kF2) continue;
-    fn(((long long)(kz + d.K) * d.P + (ky + d.K)) * d.M + kx, kx == 0 ? 1.0 : 2.0);
-  }
-}
-
-// Band energy E_f = sum_{0<|k|^2<=kF^2} w |u_k|^2 / (2 N^6) of the velocity `u`,
-// by one warp in a fixed order; every lane returns it.
 template <typename T>
-__device__ __forceinline__ double band_energy(const Dims& d, const typename CT<T>::type* u, double kF2, int lane) {
-  using C = typename CT<T>::type;
-  double s = 0.0;
-  for_band(d, kF2, lane, [&](long long i, double w) {
-    const C a = u[i], b = u[d.S + i], c = u[2 * d.S + i];
-    s += w * (((double)a.x * (double)a.x + (double)a.y * (double)a.y) +
-              ((double)b.x * (double)b.x + (double)b.y * (double)b.y) +
-              ((double)c.x * (double)c.x + (double)c.y * (double)c.y));
-  });
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  const double n3 = (double)d.N * d.N * d.N;
-  return s / (2.0 * n3 * n3);
-}
-
-// E_f of the state `in` and A = eps_inj / (2 E_f) (0 if E_f = 0).  One warp:
-// the band of kF = 2 has 75 candidate modes, and what bounds the kernel is the
-// latency of its loads, so they are issued together across the lanes (one
-// thread reading them in turn took 25-29 us per right-hand side at any N).
-template <typename T>
-__device__ __forceinline__ void b_famp(Dims d, const void* in_, Ctrl* ctrl, double kF2, double eps_inj, int forcing,
-                                       int step_start, int lane) {
-  using C = typename CT<T>::type;
-  const double ef = band_energy<T>(d, static_cast<const C*>(in_), kF2, lane);
-  if (lane != 0) return;
-  ctrl->Ef = ef;
-  if (step_start) ctrl->Ef_start = ef;
-  // the deterministic forcing keeps the rate of its last rescaling in A
-  if (forcing != 2) ctrl->A = (forcing == 1 && ef > 1e-300) ? eps_inj / (2.0 * ef) : 0.0;
-}
-template <typename T>
-__global__ void __launch_bounds__(32) k_famp(Dims d, const void* in_, Ctrl* ctrl, double kF2, double eps_inj,
-                                             int forcing, int step_start) {
-  b_famp<T>(d, in_, ctrl, kF2, eps_inj, forcing, step_start, threadIdx.x);
-}
-
-// The paper's deterministic forcing (section 2.3), after the last stage of a
-// step: the band 0 < |k|^2 <= kF^2 of the new state is multiplied by
-// f = sqrt(Ef0 / E_f) so that it keeps the energy Ef0 it had at the start of
-// the first step (Ef0 < 0: the target is taken from this step's start).  A
-// records the equivalent rate ln(f) / dt.  One warp, fixed order; each lane
-// rescales the modes it summed.
-template <typename T>
-__device__ __forceinline__ void b_hold(Dims d, void* u_, Ctrl* ctrl, double kF2, int lane) {
-  using C = typename CT<T>::type;
-  C* u = static_cast<C*>(u_);
-  const double ef = band_energy<T>(d, u, kF2, lane);
-  double ef0 = ctrl->Ef0;
-  if (ef0 < 0.0) ef0 = ctrl->Ef_start;
-  const double f = ef > 1e-300 ? sqrt(ef0 / ef) : 1.0;
-  for_band(d, kF2, lane, [&](long long i, double) {
-    for (int c = 0; c < 3; ++c) u[c * d.S + i] = cscale(u[c * d.S + i], (T)f);
-  });
-  __syncwarp();  // every lane has read Ef0
-  if (lane != 0) return;
-  ctrl->Ef0 = ef0;
-  ctrl->A = log(f) / ctrl->dt;
-  ctrl->Ef = ef * f * f;
-}
-template <typename T>
-__global__ void __launch_bounds__(32) k_hold(Dims d, void* u_, Ctrl* ctrl, double kF2) {
-  b_hold<T>(d, u_, ctrl, kF2, threadIdx.x);
-}
-
-// Integrating factors per axis: e(k) = exp(-nu k^2 dt / 2) (and with D), so
-// that exp(-nu |k|^2 dt/2) = e(|kx|) e(|ky|) e(|kz|).  FP64 exp, stored as T.
-template <typename T>
-__device__ __forceinline__ void b_iftab(int K, const Ctrl* ctrl, double nu, double D, T* eu, T* ep, int k) {
-  if (k > K) return;
-  const double dt = ctrl->dt;
-  eu[k] = (T)exp(-nu * (double)k * k * dt * 0.5);
-  ep[k] = (T)exp(-D * (double)k * k * dt * 0.5);
+__global__ void __launch_bounds__(32) k_hold(Dims d, void* u_, Ctrl* ctrl, int kb, int k2max) {
+  b_hold<T>(d, u_, ctrl, kb, k2max, threadIdx.x);
 }
 template <typename T>
 __global__ void k_iftab(int K, const Ctrl* ctrl, double nu, double D, T* eu, T* ep) {
   b_iftab<T>(K, ctrl, nu, D, eu, ep, blockIdx.x * blockDim.x + threadIdx.x);
 }
-
-#ifndef PSC_SHELLS_ONLY
-// dt = cfl dx / max(|u1|+|u2|+|u3|)  (Eq. 10) on every record_every-th step
-// (the step count lives on the device, so the launch sequence of a step never
-// changes and can be captured in a CUDA graph); a non-finite maximum raises the
-// instability flag and leaves dt unchanged.
-__device__ __forceinline__ void b_cfl(Ctrl* c, double cfl, double dx, int record_every) {
-  if (c->step % record_every != 0) return;
-  const double m = __longlong_as_double((long long)c->umax_bits);
-  if (!(m <= 1.7976931348623157e308)) { c->err |= 2; return; }
-  if (m > 0.0) c->dt = cfl * dx / m;
-}
-static __global__ void k_cfl(Ctrl* c, double cfl, double dx, int record_every) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  b_cfl(c, cfl, dx, record_every);
-}
-
-#endif  // PSC_SHELLS_ONLY
 
 // Fixed-order block sum of one double (every thread passes its value; the
 // result is valid in thread 0).

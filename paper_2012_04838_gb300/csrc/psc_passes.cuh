@@ -18,7 +18,7 @@
 // inverse is applied once, to the physical fields in the X pass.
 #pragma once
 
-#include "psc_common.cuh"
+#include "psc_scalars.cuh"
 
 namespace psc {
 
@@ -33,6 +33,7 @@ namespace psc {
 // created (see psc_capi.cu); FP64 uses W = 8.
 template <typename T, int N, int W> struct StridedCfg {
   static constexpr int THREADS = W * PlanD<N>::LPL;
+  static_assert(THREADS >= 32 || THREADS == 16 || THREADS == 8, "lead_force: a whole warp, or a power of two");
   // FP32: cap registers at 128 per thread so at least 512 threads fit on an SM;
   // FP64 is bound by the FP64 pipe, so it keeps its values in registers instead
   static constexpr int MINB = sizeof(T) == 8 ? 1 : (THREADS >= 512 ? 1 : 512 / THREADS);
@@ -230,7 +231,7 @@ __device__ __forceinline__ void b_zinv(const PassArgs& a, const Tctx& tcx) {
   // (input field, multiply by i kz, output stream)
   constexpr int nt = STATS ? 8 : 7;
 #pragma unroll 1
-  for (int tr = 0; tr < nt; ++tr) {
+  for (int tr = part_begin<N>(nt, share_of<N>(tcx), tcx.parts), te = part_begin<N>(nt, share_of<N>(tcx) + 1, tcx.parts); tr < te; ++tr) {
     int f, s;
     bool deriv;
     switch (tr) {
@@ -266,7 +267,9 @@ template <typename T, int N, bool STATS, int W, int KK = (N - 1) / 3, bool SHIFT
 __global__ void __launch_bounds__(StridedCfg<T, N, W>::THREADS, StridedCfg<T, N, W>::MINB)
 k_zinv(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  b_zinv<T, N, STATS, W, KK, SHIFT>(a, hw_ctx(smraw));
+  if (a.force.on && blockIdx.y == 0)
+    return lead_force<T>(a, threadIdx.y * blockDim.x + threadIdx.x, blockDim.x * blockDim.y);
+  b_zinv<T, N, STATS, W, KK, SHIFT>(a, hw_ctx(smraw, a.force.on));
 }
 
 template <typename T, int N, int YM, int W, int KK = (N - 1) / 3, bool SHIFT = false>
@@ -287,7 +290,7 @@ __device__ __forceinline__ void b_yinv(const PassArgs& a, const Tctx& tcx) {
   // (kind, s1, s2, out): kind 0 = s1, 1 = i ky s1, 2 = i ky s1 - s2
   constexpr int nt = YM == YMODE_CONVECTIVE ? 12 : YM == YMODE_STATS ? 11 : 9;
 #pragma unroll 1
-  for (int tr = 0; tr < nt; ++tr) {
+  for (int tr = part_begin<N>(nt, share_of<N>(tcx), tcx.parts), te = part_begin<N>(nt, share_of<N>(tcx) + 1, tcx.parts); tr < te; ++tr) {
     int kind, s1, s2 = 0, so;
     switch (tr) {
       case 0: kind = 0; s1 = Z_UX; so = Y_UX; break;
@@ -350,7 +353,7 @@ __device__ __forceinline__ void b_yfwd(const PassArgs& a, const Tctx& tcx) {
   const long long zs = (long long)N * P * M, ys = (long long)N * N * M;
   const C zero = mk(T(0), T(0));
 #pragma unroll 1
-  for (int s = 0; s < 4; ++s) {
+  for (int s = part_begin<N>(4, share_of<N>(tcx), tcx.parts), se = part_begin<N>(4, share_of<N>(tcx) + 1, tcx.parts); s < se; ++s) {
     strided_fft<T, N, W, -1, KK>(
         [&](int y) -> C {
           if (!act) return zero;
@@ -372,7 +375,9 @@ template <typename T, int N, int W, int KK = (N - 1) / 3, bool SHIFT = false>
 __global__ void __launch_bounds__(StridedCfg<T, N, W>::THREADS, StridedCfg<T, N, W>::MINB)
 k_yfwd(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  b_yfwd<T, N, W, KK, SHIFT>(a, hw_ctx(smraw));
+  if (a.cfl.on && blockIdx.y == 0)
+    return lead_cfl<T>(a, threadIdx.y * blockDim.x + threadIdx.x, blockDim.x * blockDim.y);
+  b_yfwd<T, N, W, KK, SHIFT>(a, hw_ctx(smraw, a.cfl.on));
 }
 
 template <typename T, int N, int W, int KK = (N - 1) / 3, bool SHIFT = false>
@@ -391,7 +396,7 @@ __device__ __forceinline__ void b_zfwd(const PassArgs& a, const Tctx& tcx) {
   const long long S = (long long)P * P * M, zs = (long long)N * P * M;
   const C zero = mk(T(0), T(0));
 #pragma unroll 1
-  for (int s = 0; s < 4; ++s) {
+  for (int s = part_begin<N>(4, share_of<N>(tcx), tcx.parts), se = part_begin<N>(4, share_of<N>(tcx) + 1, tcx.parts); s < se; ++s) {
     strided_fft<T, N, W, -1, KK>(
         [&](int z) -> C {
           if (!act) return zero;
@@ -995,15 +1000,46 @@ template <typename T, int N> struct Passes {
     }
   }
 
+  static int sm_count() {
+    static int n[64] = {0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return 152;
+    if (n[dev] == 0) {
+      int c = 0;
+      cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev);
+      n[dev] = c > 0 ? c : 152;
+    }
+    return n[dev];
+  }
+  // Shares (grid z) that the nt transforms of a strided pass are cut into.  A
+  // CTA otherwise runs them one after another, which is right where the tiles
+  // alone fill the SMs (512 threads each, what 128 registers a thread leave
+  // room for); below that the tiles occupy a part of the chip and the pass
+  // lasts as long as one CTA's chain of transforms, so the chain is shared out
+  // until the SMs are full (64^3 and below: every transform its own CTAs).
+  // With several boxes on the chip at once (PassArgs::share) their tiles count
+  // together: cutting the passes of 63 concurrent boxes up made their step 22%
+  // slower, through the twiddle tables that every CTA fills.
+  static int parts(const PassArgs& a, int tiles, int threads, int nt) {
+    if (!kSplit<N>) return 1;
+    const long long want = (long long)sm_count() * 512, have = (long long)tiles * threads * a.share;
+    const int s = have >= want ? 1 : (int)((want + have - 1) / have);
+    const int per = s >= nt ? 1 : (nt + s - 1) / s;
+    return (nt + per - 1) / per;
+  }
+  static constexpr int yinv_nt(int ym) { return ym == YMODE_CONVECTIVE ? 12 : ym == YMODE_STATS ? 11 : 9; }
   template <int W> static void zinv_w(const PassArgs& a, bool stats) {
     constexpr size_t sm = StridedSmem<T, N, W>::BYTES;
-    dim3 grid((M + W - 1) / W, P), block(W, PlanD<N>::LPL);
+    const int gx = (M + W - 1) / W;
+    const dim3 grid(gx, P + a.force.on, parts(a, gx * P, W * PlanD<N>::LPL, stats ? 8 : 7)), block(W, PlanD<N>::LPL);
     if (stats) { prep(k_zinv<T, N, true, W>, sm); k_zinv<T, N, true, W><<<grid, block, sm, a.st>>>(a); }
     else { prep(k_zinv<T, N, false, W>, sm); k_zinv<T, N, false, W><<<grid, block, sm, a.st>>>(a); }
   }
   template <int W, int YM> static void yinv_m(const PassArgs& a) {
     constexpr size_t sm = StridedSmem<T, N, W>::BYTES;
-    dim3 grid((M + W - 1) / W, N), block(W, PlanD<N>::LPL);
+    const int gx = (M + W - 1) / W;
+    const dim3 grid(gx, N, parts(a, gx * N, W * PlanD<N>::LPL, yinv_nt(YM))), block(W, PlanD<N>::LPL);
     prep(k_yinv<T, N, YM, W>, sm);
     k_yinv<T, N, YM, W><<<grid, block, sm, a.st>>>(a);
   }
@@ -1014,13 +1050,15 @@ template <typename T, int N> struct Passes {
   }
   template <int W> static void yfwd_w(const PassArgs& a) {
     constexpr size_t sm = StridedSmem<T, N, W>::BYTES;
-    dim3 grid((M + W - 1) / W, N), block(W, PlanD<N>::LPL);
+    const int gx = (M + W - 1) / W;
+    const dim3 grid(gx, N + a.cfl.on, parts(a, gx * N, W * PlanD<N>::LPL, 4)), block(W, PlanD<N>::LPL);
     prep(k_yfwd<T, N, W>, sm);
     k_yfwd<T, N, W><<<grid, block, sm, a.st>>>(a);
   }
   template <int W> static void zfwd_w(const PassArgs& a) {
     constexpr size_t sm = StridedSmem<T, N, W>::BYTES;
-    dim3 grid((M + W - 1) / W, P), block(W, PlanD<N>::LPL);
+    const int gx = (M + W - 1) / W;
+    const dim3 grid(gx, P, parts(a, gx * P, W * PlanD<N>::LPL, 4)), block(W, PlanD<N>::LPL);
     prep(k_zfwd<T, N, W>, sm);
     k_zfwd<T, N, W><<<grid, block, sm, a.st>>>(a);
   }
@@ -1056,8 +1094,11 @@ template <typename T, int N> struct Passes {
         rows = P;
       }
       if (!ok) return false;
+      constexpr int gx = (M + W - 1) / W;
+      const int lead = PASS == SP_ZINV ? a.force.on : PASS == SP_YFWD ? a.cfl.on : 0;
+      const dim3 grid(gx, rows + lead, parts(a, gx * rows, W * TPL, StagedPlan<PASS, MODE>::NT));
       prep(k_strided_s<T, N, W, PASS, MODE>, TL::SMEM);
-      k_strided_s<T, N, W, PASS, MODE><<<dim3((M + W - 1) / W, rows), dim3(W, TPL), TL::SMEM, a.st>>>(a, m);
+      k_strided_s<T, N, W, PASS, MODE><<<grid, dim3(W, TPL), TL::SMEM, a.st>>>(a, m);
       return true;
     } else {
       (void)a;
@@ -1106,18 +1147,6 @@ template <typename T, int N> struct Passes {
 #define PSC_X2S 1
 #endif
   static constexpr bool X2S = PSC_X2S && X2 && N == 1024 && sizeof(T) == 4;
-  static int sm_count() {
-    static int n[64] = {0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) return 152;
-    if (n[dev] == 0) {
-      int c = 0;
-      cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev);
-      n[dev] = c > 0 ? c : 152;
-    }
-    return n[dev];
-  }
   template <int MODE> static void xpass_plain(const PassArgs& a) {
     if constexpr (XROW) {
       (void)a;
@@ -1212,17 +1241,23 @@ template <typename T, int N> struct PassesPS {
     B::prep(k, sm);
     k<<<grid, block, sm, a.st>>>(a);
   }
+  template <int W> static dim3 tiles(const PassArgs& a, int rows, int lead, int nt) {
+    const int gx = (M + W - 1) / W;
+    return dim3(gx, rows + lead, B::parts(a, gx * rows, W * PlanD<N>::LPL, nt));
+  }
   template <int W, bool STATS, bool SH> static void zinv_k(const PassArgs& a) {
-    go(k_zinv<T, N, STATS, W, KS, SH>, dim3((M + W - 1) / W, P), dim3(W, PlanD<N>::LPL), StridedSmem<T, N, W>::BYTES, a);
+    go(k_zinv<T, N, STATS, W, KS, SH>, tiles<W>(a, P, a.force.on, STATS ? 8 : 7), dim3(W, PlanD<N>::LPL),
+       StridedSmem<T, N, W>::BYTES, a);
   }
   template <int W, int YM, bool SH> static void yinv_k(const PassArgs& a) {
-    go(k_yinv<T, N, YM, W, KS, SH>, dim3((M + W - 1) / W, N), dim3(W, PlanD<N>::LPL), StridedSmem<T, N, W>::BYTES, a);
+    go(k_yinv<T, N, YM, W, KS, SH>, tiles<W>(a, N, 0, B::yinv_nt(YM)), dim3(W, PlanD<N>::LPL),
+       StridedSmem<T, N, W>::BYTES, a);
   }
   template <int W, bool SH> static void yfwd_k(const PassArgs& a) {
-    go(k_yfwd<T, N, W, KS, SH>, dim3((M + W - 1) / W, N), dim3(W, PlanD<N>::LPL), StridedSmem<T, N, W>::BYTES, a);
+    go(k_yfwd<T, N, W, KS, SH>, tiles<W>(a, N, a.cfl.on, 4), dim3(W, PlanD<N>::LPL), StridedSmem<T, N, W>::BYTES, a);
   }
   template <int W, bool SH> static void zfwd_k(const PassArgs& a) {
-    go(k_zfwd<T, N, W, KS, SH>, dim3((M + W - 1) / W, P), dim3(W, PlanD<N>::LPL), StridedSmem<T, N, W>::BYTES, a);
+    go(k_zfwd<T, N, W, KS, SH>, tiles<W>(a, P, 0, 4), dim3(W, PlanD<N>::LPL), StridedSmem<T, N, W>::BYTES, a);
   }
   // X pass over the sphere's cube: the 16-values-per-thread register pass at
   // 512 and 1024, the row X pass at 520 (no convective form there), the
@@ -1285,8 +1320,11 @@ template <typename T, int N> struct PassesPS {
         rows = P;
       }
       if (!ok) return false;
+      constexpr int gx = (M + W - 1) / W;
+      const int lead = PASS == SP_ZINV ? a.force.on : PASS == SP_YFWD ? a.cfl.on : 0;
+      const dim3 grid(gx, rows + lead, B::parts(a, gx * rows, W * TPL, StagedPlan<PASS, MODE>::NT));
       B::prep(k_strided_s<T, N, W, PASS, MODE, KS, SH>, TL::SMEM);
-      k_strided_s<T, N, W, PASS, MODE, KS, SH><<<dim3((M + W - 1) / W, rows), dim3(W, TPL), TL::SMEM, a.st>>>(a, m);
+      k_strided_s<T, N, W, PASS, MODE, KS, SH><<<grid, dim3(W, TPL), TL::SMEM, a.st>>>(a, m);
       return true;
     } else {
       (void)a;

@@ -11,7 +11,7 @@
 
 #include <cuda.h>
 
-#include "psc_common.cuh"
+#include "psc_scalars.cuh"
 
 namespace psc {
 
@@ -179,8 +179,9 @@ template <int PASS, int MODE> struct StagedPlan {
   }
 };
 
-// grid (ceil(M/W), P or N), block (W, TPL).  blockIdx.y is the fixed ky (z
-// passes) or z (y passes) of the CTA's lines.  `tm` describes the pass input:
+// grid (ceil(M/W), P or N, shares of the transforms), block (W, TPL).
+// blockIdx.y is the fixed ky (z passes) or z (y passes) of the CTA's lines,
+// after the extra first row of a launch that carries scalar work.  `tm` describes the pass input:
 //   z-inverse: compact fields, 3D {2M floats, P (ky), 4P (field, kz)}
 //   y-inverse: z-stage streams, 2D {2M, Z_NSTREAM N P}
 //   y-forward: x-pass output,   2D {2M, 4 N N}
@@ -204,8 +205,19 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
   unsigned long long* bar = reinterpret_cast<unsigned long long*>(smraw + TL::BAR_OFF);
   const int w = threadIdx.x, t = threadIdx.y;
   const bool leader = w == 0 && t == 0;
-  const int x0 = blockIdx.x * W, ix = x0 + w, row = blockIdx.y;
+  int lead = 0;
+  if constexpr (PASS == SP_ZINV) {
+    lead = a.force.on;
+    if (lead && blockIdx.y == 0) return lead_force<T>(a, t * W + w, W * TPL);
+  } else if constexpr (PASS == SP_YFWD) {
+    lead = a.cfl.on;
+    if (lead && blockIdx.y == 0) return lead_cfl<T>(a, t * W + w, W * TPL);
+  }
+  const int x0 = blockIdx.x * W, ix = x0 + w, row = blockIdx.y - lead;
   const bool act = ix < M;
+  // this CTA's share of the transforms
+  const int t0 = part_begin<N>(SPL::NT, kSplit<N> ? blockIdx.z : 0, gridDim.z),
+            t1 = part_begin<N>(SPL::NT, kSplit<N> ? blockIdx.z + 1 : 1, gridDim.z);
   // a TMA destination must be 128-byte aligned: check rather than assume
   if (smem_addr(stg) & 127u) {
     if (leader) atomicOr(&a.ctrl->err, 4);
@@ -245,15 +257,15 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
       else tma_load_3d(dst, &tm, 2 * x0, row, src * N + b * TL::BOXR, bar);
     }
   };
-  if (leader) issue(0);
+  if (leader && t0 < t1) issue(t0);
   const C zero = mk(T(0), T(0));
   const C* __restrict__ zb = static_cast<const C*>(a.zb);
   unsigned parity = 0;
 #pragma unroll 1
-  for (int tr = 0; tr < SPL::NT; ++tr) {
+  for (int tr = t0; tr < t1; ++tr) {
     int src, kind, s2, out;
     SPL::get(tr, src, kind, s2, out);
-    if (!SPL::reuses(tr)) {
+    if (tr == t0 || !SPL::reuses(tr)) {
       // every thread polls the barrier, and the CTA barrier shares the
       // outcome (a transform that reuses the staged tile has nothing to wait for)
       const bool landed = mbar_wait(bar, parity, &a.ctrl->err);
@@ -304,7 +316,7 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
     // the staging tile is free (unless the next transform reads it again), and
     // the last transform's exchange reads come before this one's writes
     __syncthreads();
-    if (leader && tr + 1 < SPL::NT && !SPL::reuses(tr + 1)) issue(tr + 1);
+    if (leader && tr + 1 < t1 && !SPL::reuses(tr + 1)) issue(tr + 1);
     if constexpr (PASS == SP_ZINV) {
       C* __restrict__ zo = static_cast<C*>(a.zb);
       strided_fft_regs<T, N, W, +1, TL::TW_SMEM, KK>(
