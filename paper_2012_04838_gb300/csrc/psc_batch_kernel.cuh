@@ -161,6 +161,7 @@ __device__ __forceinline__ void run_item(const PscBatchBox& b, int pass, int til
   a.d.N = b.N;
   a.d.K = b.K;
   a.d.M = b.M;
+  a.d.MP = b.MP;
   a.d.P = b.P;
   a.d.sph = 0;
   a.d.S = b.S;

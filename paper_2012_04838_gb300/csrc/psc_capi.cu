@@ -996,8 +996,8 @@ ProbeLayout probe_layout(const Dims& d, int fp64, long long rows) {
   auto take = [&](size_t b) { size_t r = o; o = align256(o + b); return r; };
   L.ctrl = take(sizeof(Ctrl));
   L.tw = take((size_t)d.N * cs);
-  L.yb = take((size_t)Y_NSTREAM_ROT * rows * d.M * cs);
-  L.xb = take((size_t)4 * rows * d.M * cs);
+  L.yb = take((size_t)Y_NSTREAM_ROT * rows * d.MP * cs);
+  L.xb = take((size_t)4 * rows * d.MP * cs);
   L.total = o;
   return L;
 }
@@ -1041,12 +1041,12 @@ psc_status psc_xpass_probe(int32_t N, int32_t precision, int64_t rows, void* buf
   PSC_CUDA(cudaMemcpyAsync(b + L.ctrl, &c0, sizeof(c0), cudaMemcpyHostToDevice, cs));
   if (fp64) PSC_CUDA(cudaMemcpyAsync(b + L.tw, twd.data(), twd.size() * 8, cudaMemcpyHostToDevice, cs));
   else PSC_CUDA(cudaMemcpyAsync(b + L.tw, twf.data(), twf.size() * 4, cudaMemcpyHostToDevice, cs));
-  const long long nre = 2LL * Y_NSTREAM_ROT * rows * d.M;
+  const long long nre = 2LL * Y_NSTREAM_ROT * rows * d.MP;
   const double amp = 0.05 * (double)N * N * N;
   if (fp64) k_probe_fill<double><<<152 * 8, 256, 0, cs>>>((double*)(b + L.yb), nre, amp);
   else k_probe_fill<float><<<152 * 8, 256, 0, cs>>>((float*)(b + L.yb), nre, (float)amp);
   PSC_LAUNCHED("psc_xpass_probe: fill");
-  d.ys = (long long)rows * d.M;  // the X pass reads rows and stream strides from here
+  d.ys = (long long)rows * d.MP;  // the X pass reads rows and stream strides from here
   PassArgs a;
   std::memset(&a, 0, sizeof(a));
   a.d = d;
@@ -1179,6 +1179,7 @@ static PscBatchBox box_of(psc_sim* s) {
   b.N = s->d.N;
   b.K = s->d.K;
   b.M = s->d.M;
+  b.MP = s->d.MP;
   b.P = s->d.P;
   b.S = s->d.S;
   b.zs = s->d.zs;

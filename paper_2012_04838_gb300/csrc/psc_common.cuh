@@ -82,6 +82,8 @@ template <int N> struct PlanD : Plan<N> {
   // (one length-R1 DFT each), R1 lanes the second.
   static constexpr bool WIDE = J1 > 4 || J2 > 4;
   static constexpr int LPL = WIDE ? (R1 > R2 ? R1 : R2) : TPL;  // lanes per line
+  // first- and second-step DFTs of each lane in the strided passes
+  static constexpr int SJ1 = WIDE ? 1 : J1, SJ2 = WIDE ? 1 : J2;
   static_assert(R1 * R2 == N, "plan must factor N");
   static_assert(R1 % TPL == 0 && R2 % TPL == 0, "TPL must divide both radices");
   static_assert(32 % TPL == 0, "a line's threads must sit inside one warp");

@@ -216,7 +216,7 @@ __device__ __forceinline__ C shift_out(C v, const void* phase, int k) {
 template <typename T, int N, bool STATS, int W, int KK = (N - 1) / 3, bool SHIFT = false>
 __device__ __forceinline__ void b_zinv(const PassArgs& a, const Tctx& tcx) {
   using C = typename CT<T>::type;
-  constexpr int K = KK, M = KK + 1, P = 2 * KK + 1;
+  constexpr int K = KK, M = KK + 1, P = 2 * KK + 1, MP = row_pitch(M);
   unsigned char* smraw = tcx.smem;
   C* sm = reinterpret_cast<C*>(smraw);
   const int w = tcx.tx, t = tcx.ty;
@@ -226,7 +226,7 @@ __device__ __forceinline__ void b_zinv(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT in = static_cast<const C*>(a.in);
   C* PSC_RESTRICT zb = static_cast<C*>(a.zb);
   const C* tw = strided_twiddles<T, N, W>(smraw, static_cast<const C*>(a.tw), tcx);
-  const long long S = (long long)P * P * M, zs = (long long)N * P * M;
+  const long long S = (long long)P * P * M, zs = (long long)N * P * MP;
   const C zero = mk(T(0), T(0));
   // (input field, multiply by i kz, output stream)
   constexpr int nt = STATS ? 8 : 7;
@@ -256,7 +256,7 @@ __device__ __forceinline__ void b_zinv(const PassArgs& a, const Tctx& tcx) {
         },
         [&](int z, C v) {
           if (!act) return;
-          const long long idx = s * zs + ((long long)z * P + iy) * M + ix;
+          const long long idx = s * zs + ((long long)z * P + iy) * MP + ix;
           if (PSC_OK_INDEX(idx, (long long)Z_NSTREAM * zs, a.ctrl)) zb[idx] = v;
         },
         sm, tw, t, w);
@@ -275,7 +275,7 @@ k_zinv(PassArgs a) {
 template <typename T, int N, int YM, int W, int KK = (N - 1) / 3, bool SHIFT = false>
 __device__ __forceinline__ void b_yinv(const PassArgs& a, const Tctx& tcx) {
   using C = typename CT<T>::type;
-  constexpr int K = KK, M = KK + 1, P = 2 * KK + 1;
+  constexpr int K = KK, M = KK + 1, P = 2 * KK + 1, MP = row_pitch(M);
   unsigned char* smraw = tcx.smem;
   C* sm = reinterpret_cast<C*>(smraw);
   const int w = tcx.tx, t = tcx.ty;
@@ -285,7 +285,7 @@ __device__ __forceinline__ void b_yinv(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT zb = static_cast<const C*>(a.zb);
   C* PSC_RESTRICT yb = static_cast<C*>(a.yb);
   const C* tw = strided_twiddles<T, N, W>(smraw, static_cast<const C*>(a.tw), tcx);
-  const long long zs = (long long)N * P * M, ys = (long long)N * N * M;
+  const long long zs = (long long)N * P * MP, ys = (long long)N * N * MP;
   const C zero = mk(T(0), T(0));
   // (kind, s1, s2, out): kind 0 = s1, 1 = i ky s1, 2 = i ky s1 - s2
   constexpr int nt = YM == YMODE_CONVECTIVE ? 12 : YM == YMODE_STATS ? 11 : 9;
@@ -307,12 +307,12 @@ __device__ __forceinline__ void b_yinv(const PassArgs& a, const Tctx& tcx) {
       case 10: kind = 0; s1 = Z_DZUZ; so = Y_DZUZ; break;
       default: kind = 0; s1 = Z_DZUY; so = Y_DZUY; break;
     }
-    const long long rowz = (long long)z * P * M + ix;
+    const long long rowz = (long long)z * P * MP + ix;
     strided_fft<T, N, W, +1, KK>(
         [&](int p) -> C {
           int ky;
           if (!act || !k_of_pos<N, KK>(p, ky)) return zero;
-          const long long o = rowz + (long long)(ky + K) * M;
+          const long long o = rowz + (long long)(ky + K) * MP;
           if (!PSC_OK_INDEX(s1 * zs + o, (long long)Z_NSTREAM * zs, a.ctrl)) return zero;
           const C v1 = shift_in<SHIFT, KK>(zb[s1 * zs + o], a.phase, ky);
           if (kind == 0) return v1;
@@ -323,7 +323,7 @@ __device__ __forceinline__ void b_yinv(const PassArgs& a, const Tctx& tcx) {
         },
         [&](int y, C v) {
           if (!act) return;
-          const long long idx = so * ys + ((long long)z * N + y) * M + ix;
+          const long long idx = so * ys + ((long long)z * N + y) * MP + ix;
           if (PSC_OK_INDEX(idx, (long long)Y_NSTREAM * ys, a.ctrl)) yb[idx] = v;
         },
         sm, tw, t, w);
@@ -340,7 +340,7 @@ k_yinv(PassArgs a) {
 template <typename T, int N, int W, int KK = (N - 1) / 3, bool SHIFT = false>
 __device__ __forceinline__ void b_yfwd(const PassArgs& a, const Tctx& tcx) {
   using C = typename CT<T>::type;
-  constexpr int K = KK, M = KK + 1, P = 2 * KK + 1;
+  constexpr int K = KK, M = KK + 1, P = 2 * KK + 1, MP = row_pitch(M);
   unsigned char* smraw = tcx.smem;
   C* sm = reinterpret_cast<C*>(smraw);
   const int w = tcx.tx, t = tcx.ty;
@@ -350,21 +350,21 @@ __device__ __forceinline__ void b_yfwd(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT xb = static_cast<const C*>(a.xb);
   C* PSC_RESTRICT yf = static_cast<C*>(a.yf);
   const C* tw = strided_twiddles<T, N, W>(smraw, static_cast<const C*>(a.tw), tcx);
-  const long long zs = (long long)N * P * M, ys = (long long)N * N * M;
+  const long long zs = (long long)N * P * MP, ys = (long long)N * N * MP;
   const C zero = mk(T(0), T(0));
 #pragma unroll 1
   for (int s = part_begin<N>(4, share_of<N>(tcx), tcx.parts), se = part_begin<N>(4, share_of<N>(tcx) + 1, tcx.parts); s < se; ++s) {
     strided_fft<T, N, W, -1, KK>(
         [&](int y) -> C {
           if (!act) return zero;
-          const long long idx = s * ys + ((long long)z * N + y) * M + ix;
+          const long long idx = s * ys + ((long long)z * N + y) * MP + ix;
           if (!PSC_OK_INDEX(idx, 4 * ys, a.ctrl)) return zero;
           return xb[idx];
         },
         [&](int k, C v) {
           int ky;
           if (!act || !k_of_pos<N, KK>(k, ky)) return;
-          const long long idx = s * zs + ((long long)z * P + (ky + K)) * M + ix;
+          const long long idx = s * zs + ((long long)z * P + (ky + K)) * MP + ix;
           if (PSC_OK_INDEX(idx, 4 * zs, a.ctrl)) yf[idx] = shift_out<SHIFT, KK>(v, a.phase, ky);
         },
         sm, tw, t, w);
@@ -383,7 +383,7 @@ k_yfwd(PassArgs a) {
 template <typename T, int N, int W, int KK = (N - 1) / 3, bool SHIFT = false>
 __device__ __forceinline__ void b_zfwd(const PassArgs& a, const Tctx& tcx) {
   using C = typename CT<T>::type;
-  constexpr int K = KK, M = KK + 1, P = 2 * KK + 1;
+  constexpr int K = KK, M = KK + 1, P = 2 * KK + 1, MP = row_pitch(M);
   unsigned char* smraw = tcx.smem;
   C* sm = reinterpret_cast<C*>(smraw);
   const int w = tcx.tx, t = tcx.ty;
@@ -393,14 +393,14 @@ __device__ __forceinline__ void b_zfwd(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT yf = static_cast<const C*>(a.yf);
   C* PSC_RESTRICT rb = static_cast<C*>(a.rb);
   const C* tw = strided_twiddles<T, N, W>(smraw, static_cast<const C*>(a.tw), tcx);
-  const long long S = (long long)P * P * M, zs = (long long)N * P * M;
+  const long long S = (long long)P * P * M, zs = (long long)N * P * MP;
   const C zero = mk(T(0), T(0));
 #pragma unroll 1
   for (int s = part_begin<N>(4, share_of<N>(tcx), tcx.parts), se = part_begin<N>(4, share_of<N>(tcx) + 1, tcx.parts); s < se; ++s) {
     strided_fft<T, N, W, -1, KK>(
         [&](int z) -> C {
           if (!act) return zero;
-          const long long idx = s * zs + ((long long)z * P + iy) * M + ix;
+          const long long idx = s * zs + ((long long)z * P + iy) * MP + ix;
           if (!PSC_OK_INDEX(idx, 4 * zs, a.ctrl)) return zero;
           return yf[idx];
         },
@@ -563,7 +563,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
   using C = typename CT<T>::type;
   using PL = PlanD<N>;
   using XC = XCfg<T, N>;
-  constexpr int R1 = PL::R1, R2 = PL::R2, TPL = PL::TPL, J2 = PL::J2, M = KK + 1;
+  constexpr int R1 = PL::R1, R2 = PL::R2, TPL = PL::TPL, J2 = PL::J2, MP = row_pitch(KK + 1);
   constexpr int LPW = XC::LPW;
   unsigned char* smraw = tcx.smem;
   const int lane = tcx.tx & 31, wid = tcx.tx >> 5;
@@ -585,7 +585,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
     }
     __syncthreads();
   }
-  const long long ys = (long long)N * N * M;
+  const long long ys = (long long)N * N * MP;
   const long long nlines = (long long)N * N;
   const T scale = T(1.0 / ((double)N * N * N));
   const C zero = mk(T(0), T(0));
@@ -599,7 +599,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
     const bool valid = line < nlines;
     auto Y = [&](int s, int kx) -> C {
       if (!valid) return zero;
-      const long long idx = s * ys + line * M + kx;
+      const long long idx = s * ys + line * MP + kx;
       if (!PSC_OK_INDEX(idx, (long long)Y_NSTREAM * ys, a.ctrl)) return zero;
       return yb[idx];
     };
@@ -665,7 +665,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
       xfwd<T, N, KK, SHIFT>(z,
                  [&](int kx, C X1, C X2) {
                    if (!valid) return;
-                   const long long i0 = line * M + kx;
+                   const long long i0 = line * MP + kx;
                    if (PSC_OK_INDEX(i0 + ys, 4 * ys, a.ctrl)) {
                      xb[i0] = X1;
                      xb[ys + i0] = X2;
@@ -684,7 +684,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
         xfwd<T, N, KK, SHIFT>(z,
                    [&](int kx, C X1, C X2) {
                      if (!valid) return;
-                     const long long i0 = line * M + kx;
+                     const long long i0 = line * MP + kx;
                      if (PSC_OK_INDEX(i0 + 3 * ys, 4 * ys, a.ctrl)) {
                        xb[2 * ys + i0] = X1;
                        xb[3 * ys + i0] = X2;
@@ -714,7 +714,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
       xfwd<T, N, KK, SHIFT>(z,
                  [&](int kx, C X1, C X2) {
                    if (!valid) return;
-                   const long long i0 = line * M + kx;
+                   const long long i0 = line * MP + kx;
                    if (PSC_OK_INDEX(i0 + 3 * ys, 4 * ys, a.ctrl)) {
                      xb[2 * ys + i0] = X1;
                      xb[3 * ys + i0] = X2;
@@ -741,7 +741,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
       auto store = [&](int s0) {
         return [&, s0](int kx, C X1, C X2) {
           if (!valid) return;
-          const long long i0 = line * M + kx;
+          const long long i0 = line * MP + kx;
           if (PSC_OK_INDEX(i0 + (s0 + 1) * ys, 4 * ys, a.ctrl)) {
             xb[s0 * ys + i0] = X1;
             xb[(s0 + 1) * ys + i0] = X2;
@@ -941,7 +941,7 @@ namespace psc {
 
 template <typename T, int N> struct Passes {
   static constexpr int TPL = PlanD<N>::TPL;
-  static constexpr int M = PlanD<N>::M, P = PlanD<N>::P;
+  static constexpr int M = PlanD<N>::M, P = PlanD<N>::P, MP = row_pitch(M);
   // tile widths of the two variants (v = 0, 1)
   static constexpr int WV0 = 8, WV1 = sizeof(T) == 4 ? 16 : 8;
 
@@ -1062,43 +1062,46 @@ template <typename T, int N> struct Passes {
     prep(k_zfwd<T, N, W>, sm);
     k_zfwd<T, N, W><<<grid, block, sm, a.st>>>(a);
   }
-  // variants 2 and 3: input tiles staged by TMA, 4 and 8 columns (FP32, M even)
+  // variants 2 and 3: input tiles staged by TMA, 4 and 8 columns (FP32).  The
+  // z-inverse reads compact fields, whose rows are 16-byte multiples only where M
+  // is even; the other passes read padded streams
 #ifndef PSC_STAGED
 #define PSC_STAGED 1
 #endif
   // the plan and precision allow staged variants (the row length is the caller's)
-  static constexpr bool STAGED_OK = PSC_STAGED && sizeof(T) == 4 && N >= 64 && TPL >= 4;
-  static constexpr bool STAGED = STAGED_OK && M % 2 == 0;
+  static constexpr bool STAGED_OK = PSC_STAGED && sizeof(T) == 4 && N >= 64 && (TPL >= 4 || PlanD<N>::WIDE);
+  static constexpr bool STAGED = STAGED_OK;
+  template <int PASS> static constexpr bool staged_pass() { return STAGED && (PASS != SP_ZINV || M % 2 == 0); }
   // variant 4: staged, 16 columns, for the inverse passes where it fits one CTA
   static constexpr bool STAGED16 = STAGED && StagedTile<T, N, 16, true>::SMEM <= 227 * 1024;
   static constexpr int NV = STAGED16 ? 5 : STAGED ? 4 : (WV0 != WV1 ? 2 : 1);
-  static constexpr unsigned MASK_INV = (1u << NV) - 1u;
+  static constexpr unsigned MASK_INV = (1u << NV) - 1u, MASK_ZINV = staged_pass<SP_ZINV>() ? MASK_INV : MASK_INV & 3u;
   static constexpr unsigned MASK_FWD = STAGED16 ? 0xFu : (1u << NV) - 1u;
   template <int W, int PASS, int MODE> static bool launch_s(const PassArgs& a) {
-    if constexpr (STAGED) {
+    if constexpr (staged_pass<PASS>()) {
       using TL = StagedTile<T, N, W, PASS == SP_ZINV || PASS == SP_YINV>;
       CUtensorMap m;
       bool ok;
       int rows;
       if constexpr (PASS == SP_ZINV) {
-        ok = make_row_map(&m, a.in, 3, M, P, 4LL * P, (long long)P * M, W, TL::BOXR);
+        ok = make_row_map(&m, a.in, 3, M, M, P, 4LL * P, (long long)P * M, W, TL::BOXR);
         rows = P;
       } else if constexpr (PASS == SP_YINV) {
-        ok = make_row_map(&m, a.zb, 2, M, (long long)Z_NSTREAM * N * P, 0, 0, W, TL::BOXR);
+        ok = make_row_map(&m, a.zb, 2, M, MP, (long long)Z_NSTREAM * N * P, 0, 0, W, TL::BOXR);
         rows = N;
       } else if constexpr (PASS == SP_YFWD) {
-        ok = make_row_map(&m, a.xb, 2, M, 4LL * N * N, 0, 0, W, TL::BOXR);
+        ok = make_row_map(&m, a.xb, 2, M, MP, 4LL * N * N, 0, 0, W, TL::BOXR);
         rows = N;
       } else {
-        ok = make_row_map(&m, a.yf, 3, M, P, 4LL * N, (long long)P * M, W, TL::BOXR);
+        ok = make_row_map(&m, a.yf, 3, M, MP, P, 4LL * N, (long long)P * MP, W, TL::BOXR);
         rows = P;
       }
       if (!ok) return false;
       constexpr int gx = (M + W - 1) / W;
       const int lead = PASS == SP_ZINV ? a.force.on : PASS == SP_YFWD ? a.cfl.on : 0;
-      const dim3 grid(gx, rows + lead, parts(a, gx * rows, W * TPL, StagedPlan<PASS, MODE>::NT));
+      const dim3 grid(gx, rows + lead, parts(a, gx * rows, W * PlanD<N>::LPL, StagedPlan<PASS, MODE>::NT));
       prep(k_strided_s<T, N, W, PASS, MODE>, TL::SMEM);
-      k_strided_s<T, N, W, PASS, MODE><<<grid, dim3(W, TPL), TL::SMEM, a.st>>>(a, m);
+      k_strided_s<T, N, W, PASS, MODE><<<grid, dim3(W, PlanD<N>::LPL), TL::SMEM, a.st>>>(a, m);
       return true;
     } else {
       (void)a;
@@ -1218,7 +1221,7 @@ template <typename T, int N> struct Passes {
     static const PassTable tb = {&zinv, &yinv, &xpass, &yfwd, &zfwd,
                                  xwarps(), NV,
                                  {WV0, WV1, 4, 8, 16}, {0, 0, 1, 1, 1},
-                                 {MASK_INV, MASK_INV, MASK_FWD, MASK_FWD}, XROW ? 1 : 0};
+                                 {MASK_ZINV, MASK_INV, MASK_FWD, MASK_FWD}, XROW ? 1 : 0};
     return &tb;
   }
 };
@@ -1231,7 +1234,7 @@ template <typename T, int N> struct Passes {
 template <typename T, int N> struct PassesPS {
   static constexpr int KS = sphere_storage_halfwidth(N);
   static constexpr int TPL = PlanD<N>::TPL;
-  static constexpr int M = KS + 1, P = 2 * KS + 1;
+  static constexpr int M = KS + 1, P = 2 * KS + 1, MP = row_pitch(M);
   static constexpr int WV0 = 8, WV1 = sizeof(T) == 4 ? 16 : 8;
   static constexpr int NV = WV0 != WV1 ? 2 : 1;
   static_assert(P <= N, "the sphere's cube must fit the grid");
@@ -1294,37 +1297,38 @@ template <typename T, int N> struct PassesPS {
     else a.shift ? yinv_k<W, YMODE_RHS, true>(a) : yinv_k<W, YMODE_RHS, false>(a);
   }
   // variants 2-4: input tiles staged by TMA (4, 8 and, for the inverse passes,
-  // 16 columns), where the stored cube's kx rows are 16-byte multiples
-  static constexpr bool STAGED = B::STAGED_OK && M % 2 == 0;
+  // 16 columns)
+  static constexpr bool STAGED = B::STAGED_OK;
+  template <int PASS> static constexpr bool staged_pass() { return STAGED && (PASS != SP_ZINV || M % 2 == 0); }
   static constexpr bool STAGED16 = STAGED && StagedTile<T, N, 16, true, KS>::SMEM <= 227 * 1024;
   static constexpr int NVS = STAGED16 ? 5 : STAGED ? 4 : NV;
-  static constexpr unsigned MASK_INV = (1u << NVS) - 1u;
+  static constexpr unsigned MASK_INV = (1u << NVS) - 1u, MASK_ZINV = staged_pass<SP_ZINV>() ? MASK_INV : MASK_INV & 3u;
   static constexpr unsigned MASK_FWD = STAGED16 ? 0xFu : (1u << NVS) - 1u;
   template <int W, int PASS, int MODE, bool SH> static bool launch_s(const PassArgs& a) {
-    if constexpr (STAGED) {
+    if constexpr (staged_pass<PASS>()) {
       using TL = StagedTile<T, N, W, PASS == SP_ZINV || PASS == SP_YINV, KS>;
       CUtensorMap m;
       bool ok;
       int rows;
       if constexpr (PASS == SP_ZINV) {
-        ok = make_row_map(&m, a.in, 3, M, P, 4LL * P, (long long)P * M, W, TL::BOXR);
+        ok = make_row_map(&m, a.in, 3, M, M, P, 4LL * P, (long long)P * M, W, TL::BOXR);
         rows = P;
       } else if constexpr (PASS == SP_YINV) {
-        ok = make_row_map(&m, a.zb, 2, M, (long long)Z_NSTREAM * N * P, 0, 0, W, TL::BOXR);
+        ok = make_row_map(&m, a.zb, 2, M, MP, (long long)Z_NSTREAM * N * P, 0, 0, W, TL::BOXR);
         rows = N;
       } else if constexpr (PASS == SP_YFWD) {
-        ok = make_row_map(&m, a.xb, 2, M, 4LL * N * N, 0, 0, W, TL::BOXR);
+        ok = make_row_map(&m, a.xb, 2, M, MP, 4LL * N * N, 0, 0, W, TL::BOXR);
         rows = N;
       } else {
-        ok = make_row_map(&m, a.yf, 3, M, P, 4LL * N, (long long)P * M, W, TL::BOXR);
+        ok = make_row_map(&m, a.yf, 3, M, MP, P, 4LL * N, (long long)P * MP, W, TL::BOXR);
         rows = P;
       }
       if (!ok) return false;
       constexpr int gx = (M + W - 1) / W;
       const int lead = PASS == SP_ZINV ? a.force.on : PASS == SP_YFWD ? a.cfl.on : 0;
-      const dim3 grid(gx, rows + lead, B::parts(a, gx * rows, W * TPL, StagedPlan<PASS, MODE>::NT));
+      const dim3 grid(gx, rows + lead, B::parts(a, gx * rows, W * PlanD<N>::LPL, StagedPlan<PASS, MODE>::NT));
       B::prep(k_strided_s<T, N, W, PASS, MODE, KS, SH>, TL::SMEM);
-      k_strided_s<T, N, W, PASS, MODE, KS, SH><<<grid, dim3(W, TPL), TL::SMEM, a.st>>>(a, m);
+      k_strided_s<T, N, W, PASS, MODE, KS, SH><<<grid, dim3(W, PlanD<N>::LPL), TL::SMEM, a.st>>>(a, m);
       return true;
     } else {
       (void)a;
@@ -1385,7 +1389,7 @@ template <typename T, int N> struct PassesPS {
     static const PassTable tb = {&zinv, &yinv, &xpass, &yfwd, &zfwd,
                                  B::xwarps(), NVS,
                                  {WV0, WV1, 4, 8, 16}, {0, 0, 1, 1, 1},
-                                 {MASK_INV, MASK_INV, MASK_FWD, MASK_FWD}, ROWS ? 1 : 0};
+                                 {MASK_ZINV, MASK_INV, MASK_FWD, MASK_FWD}, ROWS ? 1 : 0};
     return &tb;
   }
 };

@@ -5,8 +5,9 @@
 // requested as soon as the current one has been read into registers, so its
 // global latency overlaps the current transform's compute and stores.
 //
-// Built for FP32 where a kx row is a multiple of 16 bytes (M even), which the
-// tensor-map strides require; elsewhere the unstaged kernels run.
+// Built for FP32; the z-inverse only where a compact kx row is a multiple of 16
+// bytes (M even), which the tensor-map strides require (the streams between the
+// passes are padded to that); elsewhere the unstaged kernels run.
 #pragma once
 
 #include <cuda.h>
@@ -62,28 +63,31 @@ template <typename T, int N, int W, bool INV, int KK = (N - 1) / 3> struct Stage
   // CTAs per SM that fit its 228 KB of shared memory (1 KB reserved per CTA)
   static constexpr int FIT = fit(SMEM);
   // no more CTAs than leave every thread 128 registers
-  static constexpr int RFIT = 512 / (W * PlanD<N>::TPL) < 1 ? 1 : 512 / (W * PlanD<N>::TPL);
+  static constexpr int RFIT = 512 / (W * PlanD<N>::LPL) < 1 ? 1 : 512 / (W * PlanD<N>::LPL);
   static constexpr int MINB = FIT < 1 ? 1 : (FIT < RFIT ? FIT : RFIT);
+  static_assert(!PlanD<N>::WIDE || PlanD<N>::LPL == PlanD<N>::R2, "every lane of a wide line takes a first-step DFT");
   static_assert(BOX_BYTES % 128 == 0, "boxes start 128-byte aligned");
   static_assert(W * sizeof(C) % 16 == 0, "a box row is a multiple of 16 bytes");
 };
 
 // One length-N DFT per column from step-1 inputs already in registers:
-// in[j][n1] is line position R2 n1 + t + j TPL.  Same steps as strided_fft,
+// in[j][n1] is line position R2 n1 + t + j TPL (wide lines: lanes t < R2 hold
+// position R2 n1 + t, lanes t < R1 take the second step).  Same steps as strided_fft,
 // with the step-1 twiddles wN^(n2 k1) from the shared table of
 // strided_twiddles (TW_SMEM) or from the global table tw.  It does not end
 // with a barrier: the caller's next CTA barrier must come before the exchange
 // buffer is written again.
 template <typename T, int N, int W, int DIR, bool TW_SMEM, int KK, class ST>
-__device__ __forceinline__ void strided_fft_regs(typename CT<T>::type (&in)[PlanD<N>::J1][PlanD<N>::R1],
+__device__ __forceinline__ void strided_fft_regs(typename CT<T>::type (&in)[PlanD<N>::SJ1][PlanD<N>::R1],
                                                  const ST& st, typename CT<T>::type* sm,
                                                  const typename CT<T>::type* __restrict__ tw, int t, int w) {
   using C = typename CT<T>::type;
   using PL = PlanD<N>;
   using SM = StridedSmem<T, N, W>;
-  constexpr int R1 = PL::R1, R2 = PL::R2, TPL = PL::TPL, J1 = PL::J1, J2 = PL::J2;
+  constexpr int R1 = PL::R1, R2 = PL::R2, TPL = PL::TPL;
+  constexpr int NJ1 = PL::SJ1, NJ2 = PL::SJ2;
 #pragma unroll
-  for (int j = 0; j < J1; ++j) {
+  for (int j = 0; j < NJ1; ++j) {
     const int n2 = t + j * TPL;
     first_dft<T, N, DIR, KK>(in[j]);
 #pragma unroll
@@ -91,7 +95,7 @@ __device__ __forceinline__ void strided_fft_regs(typename CT<T>::type (&in)[Plan
       C v = in[j][k1];
       if (k1 > 0) {
         // wN^(n2 k1), n2 k1 < N
-        const C wv = TW_SMEM ? tw[(j * R1 + k1) * TPL + t] : __ldg(&tw[n2 * k1]);
+        const C wv = !TW_SMEM ? __ldg(&tw[n2 * k1]) : PL::WIDE ? tw[n2 * k1] : tw[(j * R1 + k1) * TPL + t];
         v = (DIR < 0) ? cmul(v, wv) : cmulc(v, wv);
       }
       sm[k1 * SM::ROW + n2 * W + w] = v;
@@ -99,8 +103,9 @@ __device__ __forceinline__ void strided_fft_regs(typename CT<T>::type (&in)[Plan
   }
   __syncthreads();
 #pragma unroll
-  for (int j = 0; j < J2; ++j) {
+  for (int j = 0; j < NJ2; ++j) {
     const int k1 = t + j * TPL;
+    if (PL::WIDE && PL::LPL > R1 && t >= R1) break;
     C b[R2];
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) b[n2] = sm[k1 * SM::ROW + n2 * W + w];
@@ -179,7 +184,7 @@ template <int PASS, int MODE> struct StagedPlan {
   }
 };
 
-// grid (ceil(M/W), P or N, shares of the transforms), block (W, TPL).
+// grid (ceil(M/W), P or N, shares of the transforms), block (W, LPL).
 // blockIdx.y is the fixed ky (z passes) or z (y passes) of the CTA's lines,
 // after the extra first row of a launch that carries scalar work.  `tm` describes the pass input:
 //   z-inverse: compact fields, 3D {2M floats, P (ky), 4P (field, kz)}
@@ -190,7 +195,7 @@ template <int PASS, int MODE> struct StagedPlan {
 // phase-shift sphere); SHIFT: the inputs are multiplied by exp(i k pi / N) and
 // the outputs by its conjugate (the grid shifted by half a cell).
 template <typename T, int N, int W, int PASS, int MODE, int KK = (N - 1) / 3, bool SHIFT = false>
-__global__ void __launch_bounds__(W * PlanD<N>::TPL,
+__global__ void __launch_bounds__(W * PlanD<N>::LPL,
                                   StagedTile<T, N, W, PASS == SP_ZINV || PASS == SP_YINV, KK>::MINB)
 k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
   using C = typename CT<T>::type;
@@ -198,7 +203,7 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
   constexpr bool INV = PASS == SP_ZINV || PASS == SP_YINV;
   using TL = StagedTile<T, N, W, INV, KK>;
   using SPL = StagedPlan<PASS, MODE>;
-  constexpr int K = KK, M = KK + 1, P = 2 * KK + 1, R1 = PL::R1, R2 = PL::R2, TPL = PL::TPL, J1 = PL::J1;
+  constexpr int K = KK, M = KK + 1, MP = row_pitch(M), P = 2 * KK + 1, R1 = PL::R1, R2 = PL::R2, TPL = PL::TPL, NJ1 = PlanD<N>::SJ1;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   C* stg = reinterpret_cast<C*>(smraw + TL::STG_OFF);
@@ -208,10 +213,10 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
   int lead = 0;
   if constexpr (PASS == SP_ZINV) {
     lead = a.force.on;
-    if (lead && blockIdx.y == 0) return lead_force<T>(a, t * W + w, W * TPL);
+    if (lead && blockIdx.y == 0) return lead_force<T>(a, t * W + w, W * PL::LPL);
   } else if constexpr (PASS == SP_YFWD) {
     lead = a.cfl.on;
-    if (lead && blockIdx.y == 0) return lead_cfl<T>(a, t * W + w, W * TPL);
+    if (lead && blockIdx.y == 0) return lead_cfl<T>(a, t * W + w, W * PL::LPL);
   }
   const int x0 = blockIdx.x * W, ix = x0 + w, row = blockIdx.y - lead;
   const bool act = ix < M;
@@ -234,15 +239,19 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
     const C* __restrict__ g = static_cast<const C*>(a.tw);
     const int nthr = blockDim.x * blockDim.y, me = threadIdx.y * blockDim.x + threadIdx.x;
     for (int i = me; i < N; i += nthr) {
-      const int tt = i % TPL, k1 = (i / TPL) % R1, j = i / (TPL * R1);
-      t1[i] = g[(tt + j * TPL) * k1];
+      if constexpr (PL::WIDE) {
+        t1[i] = g[i];  // wide lines index wN^(n2 k1) directly
+      } else {
+        const int tt = i % TPL, k1 = (i / TPL) % R1, j = i / (TPL * R1);
+        t1[i] = g[(tt + j * TPL) * k1];
+      }
     }
     tw = t1;
   } else {
     tw = static_cast<const C*>(a.tw);
   }
   __syncthreads();  // barrier initialised and twiddles in place before use
-  const long long S = (long long)P * P * M, zs = (long long)N * P * M, ys = (long long)N * N * M;
+  const long long S = (long long)P * P * M, zs = (long long)N * P * MP, ys = (long long)N * N * MP;
   auto issue = [&](int tr) {
     int src, kind, s2, out;
     SPL::get(tr, src, kind, s2, out);
@@ -280,9 +289,9 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
       }
       parity ^= 1u;
     }
-    C in[J1][R1];
+    C in[NJ1][R1];
 #pragma unroll
-    for (int j = 0; j < J1; ++j)
+    for (int j = 0; j < NJ1; ++j)
       static_for<0, R1>([&](auto nc) {
         constexpr int n1 = decltype(nc)::value;
         const int p = R2 * n1 + t + j * TPL;
@@ -302,7 +311,7 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
                 in[j][n1] = d;
               } else {
                 // second source of omega_x, read directly (y-inverse only)
-                const long long o = s2 * zs + ((long long)row * P + (k + K)) * M + ix;
+                const long long o = s2 * zs + ((long long)row * P + (k + K)) * MP + ix;
                 in[j][n1] = PSC_OK_INDEX(o, (long long)Z_NSTREAM * zs, a.ctrl)
                                 ? csub(d, shift_in<SHIFT, KK>(zb[o], a.phase, k))
                                 : zero;
@@ -323,7 +332,7 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
           in,
           [&](int z, C v) {
             if (!act) return;
-            const long long idx = out * zs + ((long long)z * P + row) * M + ix;
+            const long long idx = out * zs + ((long long)z * P + row) * MP + ix;
             if (PSC_OK_INDEX(idx, (long long)Z_NSTREAM * zs, a.ctrl)) zo[idx] = v;
           },
           sm, tw, t, w);
@@ -333,7 +342,7 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
           in,
           [&](int y, C v) {
             if (!act) return;
-            const long long idx = out * ys + ((long long)row * N + y) * M + ix;
+            const long long idx = out * ys + ((long long)row * N + y) * MP + ix;
             if (PSC_OK_INDEX(idx, (long long)Y_NSTREAM * ys, a.ctrl)) yo[idx] = v;
           },
           sm, tw, t, w);
@@ -344,7 +353,7 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
           [&](int k, C v) {
             int ky;
             if (!act || !k_of_pos<N, KK>(k, ky)) return;
-            const long long idx = out * zs + ((long long)row * P + (ky + K)) * M + ix;
+            const long long idx = out * zs + ((long long)row * P + (ky + K)) * MP + ix;
             if (PSC_OK_INDEX(idx, 4 * zs, a.ctrl)) yo[idx] = shift_out<SHIFT, KK>(v, a.phase, ky);
           },
           sm, tw, t, w);
@@ -385,15 +394,15 @@ inline EncodeTiledFn encode_tiled_fn() {
   return fn;
 }
 
-// FP32 view of rows of M complex values: dims {2M, d1[, d2]}, row stride M
-// complex, plane stride P M complex (rank 3); boxes of {2W, 1, boxr} (rank 3)
+// FP32 view of rows of M complex values: dims {2M, d1[, d2]}, row stride
+// `pitch` and plane stride `plane` complex values (rank 3); boxes of {2W, 1, boxr} (rank 3)
 // or {2W, boxr} (rank 2).  False if the map cannot be made.
-inline bool make_row_map(CUtensorMap* m, const void* base, int rank, int M, long long d1, long long d2,
+inline bool make_row_map(CUtensorMap* m, const void* base, int rank, int M, int pitch, long long d1, long long d2,
                          long long plane, int W, int boxr) {
   EncodeTiledFn fn = encode_tiled_fn();
-  if (!fn || ((uintptr_t)base & 15) != 0 || (M * 8) % 16 != 0) return false;
+  if (!fn || ((uintptr_t)base & 15) != 0 || (pitch * 8) % 16 != 0) return false;
   cuuint64_t dims[3] = {(cuuint64_t)(2 * M), (cuuint64_t)d1, (cuuint64_t)d2};
-  cuuint64_t strides[2] = {(cuuint64_t)M * 8, (cuuint64_t)plane * 8};
+  cuuint64_t strides[2] = {(cuuint64_t)pitch * 8, (cuuint64_t)plane * 8};
   cuuint32_t box[3], es[3] = {1, 1, 1};
   box[0] = (cuuint32_t)(2 * W);
   if (rank == 3) {

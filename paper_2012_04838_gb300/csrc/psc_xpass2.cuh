@@ -323,7 +323,7 @@ __device__ __forceinline__ bool x2_rhs_row(const YF& Y, const HA& after_a, const
                                            T scale, bool want_umax, T& um, Ctrl* ctrl,
                                            const void* phase = nullptr) {
   using C = typename CT<T>::type;
-  constexpr int M = KK + 1;
+  constexpr int MP = row_pitch(KK + 1);
   const C zero = mk(T(0), T(0));
   (void)ctrl;
   C z[16];
@@ -360,7 +360,7 @@ __device__ __forceinline__ bool x2_rhs_row(const YF& Y, const HA& after_a, const
   }
   x2fwd<T, N, KK, SHIFT>(z,
               [&](int kx, C X1, C X2) {
-                const long long i0 = line * M + kx;
+                const long long i0 = line * MP + kx;
                 if (PSC_OK_INDEX(i0 + ys, 4 * ys, ctrl)) { xb[i0] = X1; xb[i0 + ys] = X2; }
               },
               ex, q, phase);
@@ -371,7 +371,7 @@ __device__ __forceinline__ bool x2_rhs_row(const YF& Y, const HA& after_a, const
       z[b] = mk(W[b] * s2, T(0.5) * (u1[b] * u1[b] + u2[b] * u2[b] + u3[b] * u3[b]) * s2);
     x2fwd<T, N, KK, SHIFT>(z,
                 [&](int kx, C X1, C X2) {
-                  const long long i0 = 2 * ys + line * M + kx;
+                  const long long i0 = 2 * ys + line * MP + kx;
                   if (PSC_OK_INDEX(i0 + ys, 4 * ys, ctrl)) { xb[i0] = X1; xb[i0 + ys] = X2; }
                 },
                 ex, q, phase);
@@ -390,7 +390,7 @@ __device__ __forceinline__ bool x2_rhs_row(const YF& Y, const HA& after_a, const
   for (int b = 0; b < 16; ++b) z[b] = mk(W[b] * s2, (u1[b] + u3[b] * z[b].x) * s2);  // (NL3, u.grad phi)
   x2fwd<T, N, KK, SHIFT>(z,
               [&](int kx, C X1, C X2) {
-                const long long i0 = 2 * ys + line * M + kx;
+                const long long i0 = 2 * ys + line * MP + kx;
                 if (PSC_OK_INDEX(i0 + ys, 4 * ys, ctrl)) { xb[i0] = X1; xb[i0 + ys] = X2; }
               },
               ex, q, phase);
@@ -411,7 +411,7 @@ __device__ __forceinline__ bool x2_conv_row(const YF& Y, const HA& after_a, cons
                                             const X2Roles<typename CT<T>::type>& q, T scale, bool want_umax, T& um,
                                             Ctrl* ctrl, const void* phase = nullptr) {
   using C = typename CT<T>::type;
-  constexpr int M = KK + 1;
+  constexpr int MP = row_pitch(KK + 1);
   const C zero = mk(T(0), T(0));
   (void)ctrl;
   C z[16];
@@ -419,7 +419,7 @@ __device__ __forceinline__ bool x2_conv_row(const YF& Y, const HA& after_a, cons
   T u1[16], u2[16], u3[16], A[16], B[16];
   auto out = [&](int s0) {
     return [&, s0](int kx, C X1, C X2) {
-      const long long i0 = s0 * ys + line * M + kx;
+      const long long i0 = s0 * ys + line * MP + kx;
       if (PSC_OK_INDEX(i0 + ys, 4 * ys, ctrl)) { xb[i0] = X1; xb[i0 + ys] = X2; }
     };
   };
@@ -489,7 +489,7 @@ template <typename T, int N, int MODE, int KK = (N - 1) / 3, bool SHIFT = false>
 __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : PSC_X2_MINB) k_xpass2(PassArgs a) {
   using C = typename CT<T>::type;
   using XC = X2Cfg<T, N>;
-  constexpr int TH = XC::TH, G = XC::G, ROWS = XC::ROWS, M = KK + 1;
+  constexpr int TH = XC::TH, G = XC::G, ROWS = XC::ROWS, MP = row_pitch(KK + 1);
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lid = threadIdx.x / TH;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : PSC_X2_MINB) k_xpass
   x2_twiddles<T, N>(reinterpret_cast<C*>(smraw + XC::LINE_BYTES * ROWS + XC::ACC_BYTES), tw, q);
   // rows and the stream stride come from the arguments (N*N rows for a pass over the box)
   const long long ys = a.d.ys;
-  const long long nlines = ys / M;
+  const long long nlines = ys / MP;
   const T scale = T(1.0 / ((double)N * N * N));
   const C zero = mk(T(0), T(0));
   // maximum of |u1|+|u2|+|u3| over the thread's points (unscaled fields in the
@@ -518,9 +518,9 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : PSC_X2_MINB) k_xpass
 #pragma unroll 1
   for (long long base = (long long)blockIdx.x * ROWS; base < nlines; base += (long long)gridDim.x * ROWS) {
     const long long line = base + lid;  // the row count (N*N, or a probe's multiple of 64) is a multiple of ROWS
-    const C* __restrict__ row = yb + line * M;
+    const C* __restrict__ row = yb + line * MP;
     auto Y = [&](int s, int kx) -> C {
-      if (!PSC_OK_INDEX(s * ys + line * M + kx, (long long)Y_NSTREAM * ys, a.ctrl)) return zero;
+      if (!PSC_OK_INDEX(s * ys + line * MP + kx, (long long)Y_NSTREAM * ys, a.ctrl)) return zero;
       return row[s * ys + kx];
     };
     C z[16];
@@ -669,8 +669,8 @@ template <typename T, int N, int KK = (N - 1) / 3, int MODE = XMODE_RHS> struct 
 #ifndef PSC_X2S_ROWS
 #define PSC_X2S_ROWS 6
 #endif
-  static constexpr int M = KK + 1;
-  static constexpr unsigned ROW_BYTES = (unsigned)(M * sizeof(C));
+  static constexpr int MP = row_pitch(KK + 1);
+  static constexpr unsigned ROW_BYTES = (unsigned)(MP * sizeof(C));
   static constexpr size_t STAGE_BYTES = (size_t)G::SLOTS * ROW_BYTES;
   static constexpr size_t GROUP_BYTES = STAGE_BYTES + XC::LINE_BYTES;
   // rows in flight: PSC_X2S_ROWS, fewer where longer rows (more streams, or the
@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
   using G = typename SC::G;
   static_assert(SC::OK, "staged x pass: rows must be 16-byte multiples and fit shared memory");
   static_assert(MODE == XMODE_RHS || MODE == XMODE_CONVECTIVE, "staged x pass: right-hand side only");
-  constexpr int TH = XC::TH, G_ = XC::G, ROWS = SC::ROWS, M = SC::M;
+  constexpr int TH = XC::TH, G_ = XC::G, ROWS = SC::ROWS, MP = SC::MP;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lid = threadIdx.x / TH;
   X2Roles<C> q;
@@ -719,8 +719,8 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
     mbar_init_fence();
   }
   x2_twiddles<T, N>(reinterpret_cast<C*>(smraw + SC::TW_OFF), static_cast<const C*>(a.tw), q);
-  const long long ys = a.d.ys;  // N*N*M for a pass over the box
-  const long long nlines = ys / M;
+  const long long ys = a.d.ys;  // N*N*MP for a pass over the box
+  const long long nlines = ys / MP;
   const long long stride = (long long)gridDim.x * ROWS;
   const T scale = T(1.0 / ((double)N * N * N));
   const bool leader = q.tid == 0;
@@ -737,9 +737,9 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
 #pragma unroll
     for (int st = 0; st < G::SLOTS; ++st) {
       if (!((mask >> st) & 1u)) continue;
-      const long long src = st * ys + ln * M;
-      if (PSC_OK_INDEX(src + M - 1, (long long)Y_NSTREAM * ys, a.ctrl))
-        bulk_copy_g2s(stg + st * M, yb + src, SC::ROW_BYTES, bar);
+      const long long src = st * ys + ln * MP;
+      if (PSC_OK_INDEX(src + MP - 1, (long long)Y_NSTREAM * ys, a.ctrl))
+        bulk_copy_g2s(stg + st * MP, yb + src, SC::ROW_BYTES, bar);
     }
   };
   T um = T(0);
@@ -763,7 +763,7 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
     if (!ok) break;
     pa ^= 1u;
     ia = false;
-    auto Y = [&](int st, int kx) -> C { return stg[st * M + kx]; };
+    auto Y = [&](int st, int kx) -> C { return stg[st * MP + kx]; };
     auto after_a = [&] {
       if (next < nlines) {
         if (leader) issue(next, G::A, barA);

@@ -87,7 +87,7 @@ template <typename T, int N, int WR, int MODE, int KK = (N - 1) / 3, bool SHIFT 
 __global__ void __launch_bounds__(XRowSmem<T, N, WR>::THREADS, 3) k_xrow(PassArgs a) {
   using C = typename CT<T>::type;
   using XS = XRowSmem<T, N, WR>;
-  constexpr int K = KK, M = KK + 1;
+  constexpr int K = KK, MP = row_pitch(KK + 1);
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   C* tw = reinterpret_cast<C*>(smraw);
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(XRowSmem<T, N, WR>::THREADS, 3) k_xrow(PassArg
   T* buf = reinterpret_cast<T*>(myrow + XS::EX_BYTES);
   const C* __restrict__ yb = static_cast<const C*>(a.yb);
   C* __restrict__ xb = static_cast<C*>(a.xb);
-  const long long ys = (long long)N * N * M;
+  const long long ys = (long long)N * N * MP;
   const long long nrows = (long long)N * N;
   const T scale = T(1.0 / ((double)N * N * N));
   const C zero = mk(T(0), T(0));
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(XRowSmem<T, N, WR>::THREADS, 3) k_xrow(PassArg
 #pragma unroll 1
   for (long long row = (long long)blockIdx.x * WR + wid; row < nrows; row += (long long)gridDim.x * WR) {
     auto Y = [&](int s, int kx) -> C {
-      const long long idx = s * ys + row * M + kx;
+      const long long idx = s * ys + row * MP + kx;
       if (!PSC_OK_INDEX(idx, (long long)Y_NSTREAM * ys, a.ctrl)) return zero;
       return yb[idx];
     };
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(XRowSmem<T, N, WR>::THREADS, 3) k_xrow(PassArg
         const C A = mk(B(b1, kx), B(b2, kx)), Bn = mk(B(b1, kn), B(b2, kn));
         const C X1 = shift_out<SHIFT, KK>(mk(T(0.5) * (A.x + Bn.x), T(0.5) * (A.y - Bn.y)), a.phase, kx);
         const C X2 = shift_out<SHIFT, KK>(mk(T(0.5) * (A.y + Bn.y), T(0.5) * (Bn.x - A.x)), a.phase, kx);
-        const long long i0 = row * M + kx;
+        const long long i0 = row * MP + kx;
         if (PSC_OK_INDEX(i0 + (s0 + 1) * ys, 4 * ys, a.ctrl)) {
           xb[s0 * ys + i0] = X1;
           xb[(s0 + 1) * ys + i0] = X2;
