@@ -18,6 +18,8 @@
 // inverse is applied once, to the physical fields in the X pass.
 #pragma once
 
+#include <cstring>
+
 #include "psc_scalars.cuh"
 
 namespace psc {
@@ -1062,29 +1064,27 @@ template <typename T, int N> struct Passes {
     prep(k_zfwd<T, N, W>, sm);
     k_zfwd<T, N, W><<<grid, block, sm, a.st>>>(a);
   }
-  // variants 2 and 3: input tiles staged by TMA, 4 and 8 columns (FP32).  The
-  // z-inverse reads compact fields, whose rows are 16-byte multiples only where M
-  // is even; the other passes read padded streams
+  // variants 2 and 3: input tiles staged in shared memory, 4 and 8 columns (FP32)
 #ifndef PSC_STAGED
 #define PSC_STAGED 1
 #endif
   // the plan and precision allow staged variants (the row length is the caller's)
   static constexpr bool STAGED_OK = PSC_STAGED && sizeof(T) == 4 && N >= 64 && (TPL >= 4 || PlanD<N>::WIDE);
   static constexpr bool STAGED = STAGED_OK;
-  template <int PASS> static constexpr bool staged_pass() { return STAGED && (PASS != SP_ZINV || M % 2 == 0); }
   // variant 4: staged, 16 columns, for the inverse passes where it fits one CTA
   static constexpr bool STAGED16 = STAGED && StagedTile<T, N, 16, true>::SMEM <= 227 * 1024;
   static constexpr int NV = STAGED16 ? 5 : STAGED ? 4 : (WV0 != WV1 ? 2 : 1);
-  static constexpr unsigned MASK_INV = (1u << NV) - 1u, MASK_ZINV = staged_pass<SP_ZINV>() ? MASK_INV : MASK_INV & 3u;
+  static constexpr unsigned MASK_INV = (1u << NV) - 1u;
   static constexpr unsigned MASK_FWD = STAGED16 ? 0xFu : (1u << NV) - 1u;
   template <int W, int PASS, int MODE> static bool launch_s(const PassArgs& a) {
-    if constexpr (staged_pass<PASS>()) {
+    if constexpr (STAGED) {
       using TL = StagedTile<T, N, W, PASS == SP_ZINV || PASS == SP_YINV>;
       CUtensorMap m;
       bool ok;
       int rows;
       if constexpr (PASS == SP_ZINV) {
-        ok = make_row_map(&m, a.in, 3, M, M, P, 4LL * P, (long long)P * M, W, TL::BOXR);
+        if constexpr (M % 2 == 0) ok = make_row_map(&m, a.in, 3, M, M, P, 4LL * P, (long long)P * M, W, TL::BOXR);
+        else std::memset(&m, 0, sizeof(m)), ok = ((uintptr_t)a.in & 7) == 0;  // copied by the threads
         rows = P;
       } else if constexpr (PASS == SP_YINV) {
         ok = make_row_map(&m, a.zb, 2, M, MP, (long long)Z_NSTREAM * N * P, 0, 0, W, TL::BOXR);
@@ -1221,7 +1221,7 @@ template <typename T, int N> struct Passes {
     static const PassTable tb = {&zinv, &yinv, &xpass, &yfwd, &zfwd,
                                  xwarps(), NV,
                                  {WV0, WV1, 4, 8, 16}, {0, 0, 1, 1, 1},
-                                 {MASK_ZINV, MASK_INV, MASK_FWD, MASK_FWD}, XROW ? 1 : 0};
+                                 {MASK_INV, MASK_INV, MASK_FWD, MASK_FWD}, XROW ? 1 : 0};
     return &tb;
   }
 };
@@ -1299,19 +1299,19 @@ template <typename T, int N> struct PassesPS {
   // variants 2-4: input tiles staged by TMA (4, 8 and, for the inverse passes,
   // 16 columns)
   static constexpr bool STAGED = B::STAGED_OK;
-  template <int PASS> static constexpr bool staged_pass() { return STAGED && (PASS != SP_ZINV || M % 2 == 0); }
   static constexpr bool STAGED16 = STAGED && StagedTile<T, N, 16, true, KS>::SMEM <= 227 * 1024;
   static constexpr int NVS = STAGED16 ? 5 : STAGED ? 4 : NV;
-  static constexpr unsigned MASK_INV = (1u << NVS) - 1u, MASK_ZINV = staged_pass<SP_ZINV>() ? MASK_INV : MASK_INV & 3u;
+  static constexpr unsigned MASK_INV = (1u << NVS) - 1u;
   static constexpr unsigned MASK_FWD = STAGED16 ? 0xFu : (1u << NVS) - 1u;
   template <int W, int PASS, int MODE, bool SH> static bool launch_s(const PassArgs& a) {
-    if constexpr (staged_pass<PASS>()) {
+    if constexpr (STAGED) {
       using TL = StagedTile<T, N, W, PASS == SP_ZINV || PASS == SP_YINV, KS>;
       CUtensorMap m;
       bool ok;
       int rows;
       if constexpr (PASS == SP_ZINV) {
-        ok = make_row_map(&m, a.in, 3, M, M, P, 4LL * P, (long long)P * M, W, TL::BOXR);
+        if constexpr (M % 2 == 0) ok = make_row_map(&m, a.in, 3, M, M, P, 4LL * P, (long long)P * M, W, TL::BOXR);
+        else std::memset(&m, 0, sizeof(m)), ok = ((uintptr_t)a.in & 7) == 0;  // copied by the threads
         rows = P;
       } else if constexpr (PASS == SP_YINV) {
         ok = make_row_map(&m, a.zb, 2, M, MP, (long long)Z_NSTREAM * N * P, 0, 0, W, TL::BOXR);
@@ -1389,7 +1389,7 @@ template <typename T, int N> struct PassesPS {
     static const PassTable tb = {&zinv, &yinv, &xpass, &yfwd, &zfwd,
                                  B::xwarps(), NVS,
                                  {WV0, WV1, 4, 8, 16}, {0, 0, 1, 1, 1},
-                                 {MASK_ZINV, MASK_INV, MASK_FWD, MASK_FWD}, ROWS ? 1 : 0};
+                                 {MASK_INV, MASK_INV, MASK_FWD, MASK_FWD}, ROWS ? 1 : 0};
     return &tb;
   }
 };

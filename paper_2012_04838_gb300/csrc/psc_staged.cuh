@@ -5,9 +5,10 @@
 // requested as soon as the current one has been read into registers, so its
 // global latency overlaps the current transform's compute and stores.
 //
-// Built for FP32; the z-inverse only where a compact kx row is a multiple of 16
-// bytes (M even), which the tensor-map strides require (the streams between the
-// passes are padded to that); elsewhere the unstaged kernels run.
+// Built for FP32.  The streams between the passes are padded so that a kx row is
+// a multiple of 16 bytes, which the tensor-map strides require; the compact
+// fields the z-inverse reads are not, and where M is odd its threads copy the
+// tile with cp.async instead (512^3: 1.28 ms a launch unstaged, 0.64 ms staged).
 #pragma once
 
 #include <cuda.h>
@@ -62,8 +63,14 @@ template <typename T, int N, int W, bool INV, int KK = (N - 1) / 3> struct Stage
   static constexpr size_t SMEM = BAR_OFF + sizeof(unsigned long long);
   // CTAs per SM that fit its 228 KB of shared memory (1 KB reserved per CTA)
   static constexpr int FIT = fit(SMEM);
-  // no more CTAs than leave every thread 128 registers
-  static constexpr int RFIT = 512 / (W * PlanD<N>::LPL) < 1 ? 1 : 512 / (W * PlanD<N>::LPL);
+  // Threads per SM the registers are shared out for: 512 (128 registers each)
+  // where a thread holds more than 16 values; the inverse passes with at most
+  // 16 run in 72 registers, and their stalls are waits for memory and shared
+  // memory, so more warps help (256^3, threads 512 / 640 / 768 / 896: z-inverse
+  // 74 / 71 / 69 / 65 us, y-inverse 158 / 142 / 142 / 132; the forward passes lose
+  // 5% at 640 and above)
+  static constexpr int THREADS_SM = INV && N / PlanD<N>::TPL <= 16 ? 896 : 512;
+  static constexpr int RFIT = THREADS_SM / (W * PlanD<N>::LPL) < 1 ? 1 : THREADS_SM / (W * PlanD<N>::LPL);
   static constexpr int MINB = FIT < 1 ? 1 : (FIT < RFIT ? FIT : RFIT);
   static_assert(!PlanD<N>::WIDE || PlanD<N>::LPL == PlanD<N>::R2, "every lane of a wide line takes a first-step DFT");
   static_assert(BOX_BYTES % 128 == 0, "boxes start 128-byte aligned");
@@ -210,6 +217,9 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
   unsigned long long* bar = reinterpret_cast<unsigned long long*>(smraw + TL::BAR_OFF);
   const int w = threadIdx.x, t = threadIdx.y;
   const bool leader = w == 0 && t == 0;
+  // compact rows of odd length (z-inverse) have no tensor map: the threads copy
+  // the tile with 8-byte asynchronous copies that arrive on the same mbarrier
+  constexpr bool CPA = PASS == SP_ZINV && M % 2 != 0;
   int lead = 0;
   if constexpr (PASS == SP_ZINV) {
     lead = a.force.on;
@@ -229,7 +239,7 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
     return;
   }
   if (leader) {
-    mbar_init(bar, 1);
+    mbar_init(bar, CPA ? W * PL::LPL : 1);
     mbar_init_fence();
   }
   const C* tw;
@@ -252,9 +262,21 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
   }
   __syncthreads();  // barrier initialised and twiddles in place before use
   const long long S = (long long)P * P * M, zs = (long long)N * P * MP, ys = (long long)N * N * MP;
+  const C* __restrict__ cin = static_cast<const C*>(a.in);
   auto issue = [&](int tr) {
     int src, kind, s2, out;
     SPL::get(tr, src, kind, s2, out);
+    if constexpr (CPA) {
+      // every thread copies its column's share of the P runs
+      if (act) {
+        const C* __restrict__ g = cin + ((long long)src * P * P + row) * M + ix;
+        for (int k = t; k < P; k += PL::LPL)
+          if (PSC_OK_INDEX(((long long)src * P * P + row + (long long)k * P) * M + ix, 4 * S, a.ctrl))
+            cp_async_8(stg + k * W + w, g + (long long)k * P * M);
+      }
+      cp_async_arrive(bar);
+      return;
+    }
     fence_proxy_async_smem();
     mbar_expect_tx(bar, TL::BYTES);
 #pragma unroll
@@ -266,7 +288,7 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
       else tma_load_3d(dst, &tm, 2 * x0, row, src * N + b * TL::BOXR, bar);
     }
   };
-  if (leader && t0 < t1) issue(t0);
+  if ((CPA || leader) && t0 < t1) issue(t0);
   const C zero = mk(T(0), T(0));
   const C* __restrict__ zb = static_cast<const C*>(a.zb);
   unsigned parity = 0;
@@ -281,10 +303,8 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
       if (!__syncthreads_and(landed)) {
         // the tile did not arrive in time: report, give it a bounded time to
         // land in this CTA's shared memory, and stop
-        if (leader) {
-          atomicOr(&a.ctrl->err, 4);
-          mbar_wait(bar, parity);
-        }
+        if (leader) atomicOr(&a.ctrl->err, 4);
+        if (CPA || leader) mbar_wait(bar, parity);
         return;
       }
       parity ^= 1u;
@@ -325,7 +345,7 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
     // the staging tile is free (unless the next transform reads it again), and
     // the last transform's exchange reads come before this one's writes
     __syncthreads();
-    if (leader && tr + 1 < t1 && !SPL::reuses(tr + 1)) issue(tr + 1);
+    if ((CPA || leader) && tr + 1 < t1 && !SPL::reuses(tr + 1)) issue(tr + 1);
     if constexpr (PASS == SP_ZINV) {
       C* __restrict__ zo = static_cast<C*>(a.zb);
       strided_fft_regs<T, N, W, +1, TL::TW_SMEM, KK>(
