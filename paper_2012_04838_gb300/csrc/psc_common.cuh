@@ -40,6 +40,10 @@ __device__ __forceinline__ float2 mul_ik(float2 a, float k) {
 __device__ __forceinline__ double2 mul_ik(double2 a, double k) {
   return make_double2(__dmul_rn(-k, a.y), __dmul_rn(k, a.x));
 }
+// a b - c d and a b + c d, one product rounded and the other fused (the same
+// reason: every X pass forms the products of the right-hand side this way)
+template <typename T> __device__ __forceinline__ T det2(T a, T b, T c, T d) { return fma(a, b, -fmul_exact_order(c, d)); }
+template <typename T> __device__ __forceinline__ T dot2(T a, T b, T c, T d) { return fma(a, b, fmul_exact_order(c, d)); }
 template <class C> __device__ __forceinline__ C cadd(C a, C b) { return mk(a.x + b.x, a.y + b.y); }
 template <class C> __device__ __forceinline__ C csub(C a, C b) { return mk(a.x - b.x, a.y - b.y); }
 template <class C, typename T> __device__ __forceinline__ C cscale(C a, T s) {

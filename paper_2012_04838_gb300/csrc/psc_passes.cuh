@@ -448,12 +448,21 @@ template <typename T, int N> struct XCfg {
   static constexpr size_t SMEM = LINE_BYTES * LPW * WARPS + TW_BYTES;
 };
 
+// Positions s0 .. s0 + w - 1 of a length-N axis truncated to |k| <= K: 1 if all
+// are retained, 0 if none is, 2 if mixed.
+__host__ __device__ constexpr int slot_band(int N, int s0, int w, int K) {
+  return (s0 + w - 1 <= K || s0 >= N - K) ? 1 : (s0 > K && s0 + w - 1 < N - K) ? 0 : 2;
+}
+
 // Inverse DFT of one row from its half spectrum, two real fields at once:
 // Z[p] = X1[p] + i X2[p] (p <= K; imaginary parts dropped at p = 0),
 // conj(X1[N-p]) + i conj(X2[N-p]) (p >= N-K), 0 elsewhere.  On return
 // z[j][k2] holds scale * IDFT(Z) at position (t + j TPL) + R1 k2, whose real
-// and imaginary parts are the two real fields.
-template <typename T, int N, int KK = (N - 1) / 3, bool SHIFT = false, class SPEC>
+// and imaginary parts are the two real fields (SCALE = false: the unscaled
+// IDFT; the caller folds 1/N^3 into its products).  A slot's TPL positions lie
+// on adjacent lanes, so which slots are retained, zero or mixed is known when
+// the kernel is compiled: zero slots are neither read nor transformed.
+template <typename T, int N, bool SCALE, int KK = (N - 1) / 3, bool SHIFT = false, class SPEC>
 __device__ __forceinline__ void xinv(const SPEC& spec,
                                      typename CT<T>::type (&z)[PlanD<N>::J2][PlanD<N>::R2],
                                      typename CT<T>::type* ex,
@@ -463,37 +472,48 @@ __device__ __forceinline__ void xinv(const SPEC& spec,
   using PL = PlanD<N>;
   using XC = XCfg<T, N>;
   constexpr int R1 = PL::R1, R2 = PL::R2, TPL = PL::TPL, K = KK;
-#pragma unroll
-  for (int j = 0; j < PL::J1; ++j) {
+  static_for<0, PL::J1>([&](auto jc) {
+    constexpr int j = decltype(jc)::value;
     const int n2 = t + j * TPL;
     C a[R1];
-#pragma unroll
-    for (int n1 = 0; n1 < R1; ++n1) {
-      const int p = R2 * n1 + n2;
+    static_for<0, R1>([&](auto nc) {
+      constexpr int n1 = decltype(nc)::value;
+      constexpr int s0 = R2 * n1 + j * TPL;
+      constexpr int band = slot_band(N, s0, TPL, K);
+      const int p = s0 + t;
       C x1, x2;
-      if (p <= K) {
+      auto low = [&]() {
         spec(p, x1, x2);
         x1 = shift_in<SHIFT, KK>(x1, phase, p);
         x2 = shift_in<SHIFT, KK>(x2, phase, p);
-        if (p == 0) { x1.y = T(0); x2.y = T(0); }
+        if (s0 == 0 && p == 0) { x1.y = T(0); x2.y = T(0); }
         a[n1] = mk(x1.x - x2.y, x1.y + x2.x);
-      } else if (p >= N - K) {
+      };
+      auto high = [&]() {
         spec(N - p, x1, x2);
         x1 = shift_in<SHIFT, KK>(x1, phase, N - p);
         x2 = shift_in<SHIFT, KK>(x2, phase, N - p);
         a[n1] = mk(x1.x + x2.y, x2.x - x1.y);
+      };
+      if constexpr (band == 0) {
+        a[n1] = mk(T(0), T(0));
+      } else if constexpr (band == 1) {
+        if constexpr (s0 <= K) low();
+        else high();
       } else {
         a[n1] = mk(T(0), T(0));
+        if (s0 <= K && p <= K) low();
+        else if (s0 + TPL > N - K && p >= N - K) high();
       }
-    }
-    Dft<R1, +1>::template run<T, C>(a);
+    });
+    first_dft<T, N, +1, KK>(a);
 #pragma unroll
     for (int k1 = 0; k1 < R1; ++k1) {
       C v = a[k1];
       if (k1 > 0) v = cmulc(v, tw[(j * R1 + k1) * TPL + t]);  // wN^(-n2 k1)
       ex[k1 * XC::ROWI + n2] = v;
     }
-  }
+  });
   __syncwarp();
 #pragma unroll
   for (int j = 0; j < PL::J2; ++j) {
@@ -501,8 +521,10 @@ __device__ __forceinline__ void xinv(const SPEC& spec,
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) z[j][n2] = ex[k1 * XC::ROWI + n2];
     Dft<R2, +1>::template run<T, C>(z[j]);
+    if constexpr (SCALE) {
 #pragma unroll
-    for (int k2 = 0; k2 < R2; ++k2) z[j][k2] = cscale(z[j][k2], scale);
+      for (int k2 = 0; k2 < R2; ++k2) z[j][k2] = cscale(z[j][k2], scale);
+    }
   }
   __syncwarp();
 }
@@ -510,6 +532,7 @@ __device__ __forceinline__ void xinv(const SPEC& spec,
 // Forward DFT of a row holding two real fields packed as x1 + i x2 at the
 // positions xinv leaves them in; out(kx, X1, X2) receives both half spectra
 // for kx <= K: X1 = (Z[k] + conj Z[N-k])/2, X2 = (Z[k] - conj Z[N-k])/(2i).
+// Output slots that no kx keeps are not stored, and so not computed.
 template <typename T, int N, int KK = (N - 1) / 3, bool SHIFT = false, class OUT>
 __device__ __forceinline__ void xfwd(typename CT<T>::type (&x)[PlanD<N>::J2][PlanD<N>::R2],
                                      const OUT& out, typename CT<T>::type* ex,
@@ -540,12 +563,13 @@ __device__ __forceinline__ void xfwd(typename CT<T>::type (&x)[PlanD<N>::J2][Pla
     Dft<R1, -1>::template run<T, C>(b[j]);
   }
   __syncwarp();
-#pragma unroll
-  for (int j = 0; j < PL::J1; ++j) {
-    const int k1 = t + j * TPL;
-#pragma unroll
-    for (int k2 = 0; k2 < R1; ++k2) ex[k1 + R2 * k2] = b[j][k2];
-  }
+  static_for<0, PL::J1>([&](auto jc) {
+    constexpr int j = decltype(jc)::value;
+    static_for<0, R1>([&](auto kc) {
+      constexpr int k2 = decltype(kc)::value;
+      if constexpr (slot_band(N, j * TPL + R2 * k2, TPL, K) != 0) ex[t + j * TPL + R2 * k2] = b[j][k2];
+    });
+  });
   __syncwarp();
   for (int kx = t; kx <= K; kx += TPL) {
     const C A = ex[kx];
@@ -587,36 +611,55 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
     }
     __syncthreads();
   }
-  const long long ys = (long long)N * N * MP;
-  const long long nlines = (long long)N * N;
+  constexpr long long ys = (long long)N * N * MP;
+  constexpr long long nlines = (long long)N * N;
+  // every group of a warp is full: no row needs a bounds test
+  constexpr bool FULL = nlines % LPW == 0;
   const T scale = T(1.0 / ((double)N * N * N));
+  // the inverse transforms of the right-hand side are left unscaled (N^3 times
+  // the fields); each product carries the missing 1/N^6 once
+  const T s2 = scale * scale;
   const C zero = mk(T(0), T(0));
-  T um = T(0);  // maximum of |u1|+|u2|+|u3| over the thread's points
+  // maximum of |u1|+|u2|+|u3| over the thread's points (unscaled fields in the
+  // right-hand side, scaled in the statistics)
+  T um = T(0);
   MomentSum<T> acc[MODE == XMODE_STATS ? NQ : 1];
 
 #pragma unroll 1
   for (long long grp = (long long)tcx.bx * XC::WARPS + wid; grp * LPW < nlines;
        grp += (long long)tcx.gdx * XC::WARPS) {
     const long long line = grp * LPW + g;
-    const bool valid = line < nlines;
+    const bool valid = FULL || line < nlines;
+    const C* PSC_RESTRICT row = yb + line * MP;
+    C* PSC_RESTRICT orow = xb + line * MP;
     auto Y = [&](int s, int kx) -> C {
       if (!valid) return zero;
-      const long long idx = s * ys + line * MP + kx;
-      if (!PSC_OK_INDEX(idx, (long long)Y_NSTREAM * ys, a.ctrl)) return zero;
-      return yb[idx];
+      if (!PSC_OK_INDEX(s * ys + line * MP + kx, (long long)Y_NSTREAM * ys, a.ctrl)) return zero;
+      return row[s * ys + kx];
+    };
+    // outputs of one forward transform: streams s0 and s0 + 1
+    auto store = [&](int s0) {
+      return [&, s0](int kx, C X1, C X2) {
+        if (!valid) return;
+        if (PSC_OK_INDEX((s0 + 1) * ys + line * MP + kx, 4 * ys, a.ctrl)) {
+          orow[s0 * ys + kx] = X1;
+          orow[(s0 + 1) * ys + kx] = X2;
+        }
+      };
     };
     auto pos = [&](int j, int k2) { return (t + j * TPL) + R1 * k2; };
     C z[J2][R2];
 
     if constexpr (MODE == XMODE_RHS || MODE == XMODE_PRESSURE) {
-      T ux[J2][R2], uy[J2][R2], uz[J2][R2];
-      T nlx[J2][R2], nly[J2][R2], nlz[J2][R2], sv[J2][R2];
+      // live per thread at most: u1, u2, u3 (or their slots in shared memory)
+      // and one more field beside the transform
+      T ux[J2][R2], uy[J2][R2], uz[J2][R2], W[J2][R2];
       auto getu = [&](int c, int j, int k2) -> T {
         if constexpr (XC::STASH) return stash[c * N + pos(j, k2)];
         else return c == 0 ? ux[j][k2] : (c == 1 ? uy[j][k2] : uz[j][k2]);
       };
       // (u1, u2)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UY, kx); }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UY, kx); }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
@@ -630,20 +673,19 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
           }
         }
       // (u3, omega_1)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UZ, kx); x2 = Y(Y_WX, kx); }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UZ, kx); x2 = Y(Y_WX, kx); }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) {
-          const T u3 = z[j][k2].x, w1 = z[j][k2].y;
+          const T u3 = z[j][k2].x;
           if constexpr (XC::STASH) stash[2 * N + pos(j, k2)] = u3;
           else uz[j][k2] = u3;
-          nly[j][k2] = u3 * w1;
-          nlz[j][k2] = -getu(1, j, k2) * w1;
+          W[j][k2] = z[j][k2].y;  // omega_1
           if (a.want_umax) um = max_keep_nan(um, fabs(getu(0, j, k2)) + fabs(getu(1, j, k2)) + fabs(u3));
         }
       // (omega_2, omega_3):  omega_2 = d_z u_1 - i kx u_3,  omega_3 = i kx u_2 - d_y u_1
-      xinv<T, N, KK, SHIFT>(
+      xinv<T, N, false, KK, SHIFT>(
           [&](int kx, C& x1, C& x2) {
             x1 = csub(Y(Y_DZUX, kx), mul_ik(Y(Y_UZ, kx), T(kx)));
             x2 = csub(mul_ik(Y(Y_UY, kx), T(kx)), Y(Y_DYUX, kx));
@@ -653,27 +695,12 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) {
-          const T w2 = z[j][k2].x, w3 = z[j][k2].y;
+          const T w1 = W[j][k2], w2 = z[j][k2].x, w3 = z[j][k2].y;
           const T u1 = getu(0, j, k2), u2 = getu(1, j, k2), u3 = getu(2, j, k2);
-          nlx[j][k2] = u2 * w3 - u3 * w2;
-          nly[j][k2] -= u1 * w3;
-          nlz[j][k2] += u1 * w2;
+          z[j][k2] = mk(det2(u2, w3, u3, w2) * s2, det2(u3, w1, u1, w3) * s2);  // (NL1, NL2)
+          W[j][k2] = det2(u1, w2, u2, w1);                                      // NL3
         }
-      // forward (NL1, NL2)
-#pragma unroll
-      for (int j = 0; j < J2; ++j)
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) z[j][k2] = mk(nlx[j][k2], nly[j][k2]);
-      xfwd<T, N, KK, SHIFT>(z,
-                 [&](int kx, C X1, C X2) {
-                   if (!valid) return;
-                   const long long i0 = line * MP + kx;
-                   if (PSC_OK_INDEX(i0 + ys, 4 * ys, a.ctrl)) {
-                     xb[i0] = X1;
-                     xb[ys + i0] = X2;
-                   }
-                 },
-                 ex, tw, t, a.phase);
+      xfwd<T, N, KK, SHIFT>(z, store(0), ex, tw, t, a.phase);
       if constexpr (MODE == XMODE_PRESSURE) {
         // (NL3, |u|^2 / 2): the inputs of the modified pressure
 #pragma unroll
@@ -681,48 +708,28 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
 #pragma unroll
           for (int k2 = 0; k2 < R2; ++k2) {
             const T u1 = getu(0, j, k2), u2 = getu(1, j, k2), u3 = getu(2, j, k2);
-            z[j][k2] = mk(nlz[j][k2], T(0.5) * (u1 * u1 + u2 * u2 + u3 * u3));
+            z[j][k2] = mk(W[j][k2] * s2, T(0.5) * (u1 * u1 + u2 * u2 + u3 * u3) * s2);
           }
-        xfwd<T, N, KK, SHIFT>(z,
-                   [&](int kx, C X1, C X2) {
-                     if (!valid) return;
-                     const long long i0 = line * MP + kx;
-                     if (PSC_OK_INDEX(i0 + 3 * ys, 4 * ys, a.ctrl)) {
-                       xb[2 * ys + i0] = X1;
-                       xb[3 * ys + i0] = X2;
-                     }
-                   },
-                   ex, tw, t, a.phase);
+        xfwd<T, N, KK, SHIFT>(z, store(2), ex, tw, t, a.phase);
         continue;
       }
-      // (dphi/dx1, dphi/dx2)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); },
+      // (dphi/dx1, dphi/dx2); the slot of u1 then holds the partial u . grad phi
+      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); },
                  z, ex, tw, t, scale, a.phase);
+      T sv[J2][R2];
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2)
-          sv[j][k2] = getu(0, j, k2) * z[j][k2].x + getu(1, j, k2) * z[j][k2].y;
+          sv[j][k2] = dot2(getu(0, j, k2), z[j][k2].x, getu(1, j, k2), z[j][k2].y);
       // (dphi/dx3, 0)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) {
-          sv[j][k2] += getu(2, j, k2) * z[j][k2].x;
-          z[j][k2] = mk(nlz[j][k2], sv[j][k2]);
-        }
-      // forward (NL3, u.grad phi)
-      xfwd<T, N, KK, SHIFT>(z,
-                 [&](int kx, C X1, C X2) {
-                   if (!valid) return;
-                   const long long i0 = line * MP + kx;
-                   if (PSC_OK_INDEX(i0 + 3 * ys, 4 * ys, a.ctrl)) {
-                     xb[2 * ys + i0] = X1;
-                     xb[3 * ys + i0] = X2;
-                   }
-                 },
-                 ex, tw, t, a.phase);
+        for (int k2 = 0; k2 < R2; ++k2)
+          z[j][k2] = mk(W[j][k2] * s2, fma(getu(2, j, k2), z[j][k2].x, sv[j][k2]) * s2);  // (NL3, u.grad phi)
+      xfwd<T, N, KK, SHIFT>(z, store(2), ex, tw, t, a.phase);
     } else if constexpr (MODE == XMODE_CONVECTIVE) {
       // -(u.grad)u and u.grad phi from u, its nine gradients and grad phi; with
       // this stream set Y_WX holds d_y u_z and Y_DZUY holds d_z u_y
@@ -740,24 +747,14 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
           else uz[j][k2] = v;
         }
       };
-      auto store = [&](int s0) {
-        return [&, s0](int kx, C X1, C X2) {
-          if (!valid) return;
-          const long long i0 = line * MP + kx;
-          if (PSC_OK_INDEX(i0 + (s0 + 1) * ys, 4 * ys, a.ctrl)) {
-            xb[s0 * ys + i0] = X1;
-            xb[(s0 + 1) * ys + i0] = X2;
-          }
-        };
-      };
       // (u1, u2)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UY, kx); }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UY, kx); }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) { putu(0, j, k2, z[j][k2].x); putu(1, j, k2, z[j][k2].y); }
       // (u3, d1 u1)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UZ, kx); x2 = mul_ik(Y(Y_UX, kx), T(kx)); }, z, ex, tw, t,
+      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UZ, kx); x2 = mul_ik(Y(Y_UX, kx), T(kx)); }, z, ex, tw, t,
                  scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
@@ -768,50 +765,50 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
           if (a.want_umax) um = max_keep_nan(um, fabs(getu(0, j, k2)) + fabs(getu(1, j, k2)) + fabs(z[j][k2].x));
         }
       // (d2 u1, d3 u1): aa = (u.grad) u1
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DYUX, kx); x2 = Y(Y_DZUX, kx); }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DYUX, kx); x2 = Y(Y_DZUX, kx); }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) aa[j][k2] += getu(1, j, k2) * z[j][k2].x + getu(2, j, k2) * z[j][k2].y;
       // (d1 u2, d2 u2)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_UY, kx), T(kx)); x2 = Y(Y_DYUY, kx); }, z, ex, tw, t,
+      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_UY, kx), T(kx)); x2 = Y(Y_DYUY, kx); }, z, ex, tw, t,
                  scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) bb[j][k2] = getu(0, j, k2) * z[j][k2].x + getu(1, j, k2) * z[j][k2].y;
       // (d3 u2, d1 u3): bb = (u.grad) u2; aa starts (u.grad) u3
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZUY, kx); x2 = mul_ik(Y(Y_UZ, kx), T(kx)); }, z, ex, tw, t,
+      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZUY, kx); x2 = mul_ik(Y(Y_UZ, kx), T(kx)); }, z, ex, tw, t,
                  scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) {
           const T b2 = bb[j][k2] + getu(2, j, k2) * z[j][k2].x, c3 = getu(0, j, k2) * z[j][k2].y;
-          z[j][k2] = mk(-aa[j][k2], -b2);  // (NL1, NL2)
+          z[j][k2] = mk(-aa[j][k2] * s2, -b2 * s2);  // (NL1, NL2)
           aa[j][k2] = c3;
         }
       xfwd<T, N, KK, SHIFT>(z, store(0), ex, tw, t, a.phase);
       // (d2 u3, d3 u3): aa = (u.grad) u3
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_WX, kx); x2 = Y(Y_DZUZ, kx); }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_WX, kx); x2 = Y(Y_DZUZ, kx); }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) aa[j][k2] += getu(1, j, k2) * z[j][k2].x + getu(2, j, k2) * z[j][k2].y;
       // (dphi/dx1, dphi/dx2)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); }, z, ex, tw, t,
+      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); }, z, ex, tw, t,
                  scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) bb[j][k2] = getu(0, j, k2) * z[j][k2].x + getu(1, j, k2) * z[j][k2].y;
       // (dphi/dx3, 0)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2)
-          z[j][k2] = mk(-aa[j][k2], bb[j][k2] + getu(2, j, k2) * z[j][k2].x);  // (NL3, u.grad phi)
+          z[j][k2] = mk(-aa[j][k2] * s2, (bb[j][k2] + getu(2, j, k2) * z[j][k2].x) * s2);  // (NL3, u.grad phi)
       xfwd<T, N, KK, SHIFT>(z, store(2), ex, tw, t, a.phase);
     } else {
       // statistics: moments of the diagonal velocity gradients and the scalar
@@ -827,7 +824,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
         (void)j; (void)k2;
       };
       // (u1, u3)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UZ, kx); }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, true, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UZ, kx); }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
@@ -837,7 +834,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
           s13[j][k2] = fabs(u1) + fabs(u3);
         }
       // (u2, phi)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UY, kx); x2 = Y(Y_PHI, kx); }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, true, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UY, kx); x2 = Y(Y_PHI, kx); }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
@@ -849,7 +846,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
           um = max_keep_nan(um, s13[j][k2] + fabs(u2));
         }
       // (omega_1, omega_2)
-      xinv<T, N, KK, SHIFT>(
+      xinv<T, N, true, KK, SHIFT>(
           [&](int kx, C& x1, C& x2) {
             x1 = Y(Y_WX, kx);
             x2 = csub(Y(Y_DZUX, kx), mul_ik(Y(Y_UZ, kx), T(kx)));
@@ -861,7 +858,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
         for (int k2 = 0; k2 < R2; ++k2)
           acc[1].add(z[j][k2].x * z[j][k2].x + z[j][k2].y * z[j][k2].y);
       // (omega_3, dphi/dx1)
-      xinv<T, N, KK, SHIFT>(
+      xinv<T, N, true, KK, SHIFT>(
           [&](int kx, C& x1, C& x2) {
             x1 = csub(mul_ik(Y(Y_UY, kx), T(kx)), Y(Y_DYUX, kx));
             x2 = mul_ik(Y(Y_PHI, kx), T(kx));
@@ -875,7 +872,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
           acc234(11, j, k2, z[j][k2].y);
         }
       // (dphi/dx2, dphi/dx3)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DYPHI, kx); x2 = Y(Y_DZPHI, kx); }, z, ex, tw, t,
+      xinv<T, N, true, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DYPHI, kx); x2 = Y(Y_DZPHI, kx); }, z, ex, tw, t,
                  scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
@@ -885,7 +882,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
           acc234(17, j, k2, z[j][k2].y);
         }
       // (du1/dx1, du2/dx2)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_UX, kx), T(kx)); x2 = Y(Y_DYUY, kx); }, z,
+      xinv<T, N, true, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_UX, kx), T(kx)); x2 = Y(Y_DYUY, kx); }, z,
                  ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
@@ -895,7 +892,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
           acc234(5, j, k2, z[j][k2].y);
         }
       // (du3/dx3, 0)
-      xinv<T, N, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZUZ, kx); x2 = zero; }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, true, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZUZ, kx); x2 = zero; }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
@@ -904,7 +901,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
   }
 
   if (MODE == XMODE_STATS || a.want_umax) {
-    double umax = (double)um;  // the fields here are scaled
+    double umax = MODE == XMODE_STATS ? (double)um : (double)um * (double)scale;
     for (int o = 16; o > 0; o >>= 1) {
       const double other = __shfl_xor_sync(0xffffffffu, umax, o);
       umax = other > umax || other != other ? other : umax;
@@ -922,8 +919,17 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
   }
 }
 
+// CTAs per SM the registers are shared out for.  Left alone the compiler hoists
+// the loads of several transforms at once, up to 250 registers (the convective
+// form at 256^3 took 364 us a launch so, 318 with three CTAs).  FP64: one, it is
+// bound by the FP64 pipe.
+template <typename T, int N, int MODE, bool SPHERE> constexpr int xpass_ctas() {
+  if (sizeof(T) == 8) return 1;
+  if (XCfg<T, N>::PER <= 8) return MODE == XMODE_STATS ? 3 : 5;
+  return MODE == XMODE_STATS || (MODE == XMODE_CONVECTIVE && SPHERE) ? 2 : 3;
+}
 template <typename T, int N, int MODE, int KK = (N - 1) / 3, bool SHIFT = false>
-__global__ void __launch_bounds__(32 * XCfg<T, N>::WARPS)
+__global__ void __launch_bounds__(32 * XCfg<T, N>::WARPS, xpass_ctas<T, N, MODE, (KK > (N - 1) / 3)>())
 k_xpass(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   b_xpass<T, N, MODE, KK, SHIFT>(a, hw_ctx(smraw));
@@ -1145,11 +1151,9 @@ template <typename T, int N> struct Passes {
     if (v >= 2 && staged<SP_ZFWD>(a, 0, v)) return;
     v == 1 ? zfwd_w<WV1>(a) : zfwd_w<WV0>(a);
   }
-  // the right-hand side at N = 1024 (FP32) stages its rows through shared memory
-#ifndef PSC_X2S
-#define PSC_X2S 1
-#endif
-  static constexpr bool X2S = PSC_X2S && X2 && N == 1024 && sizeof(T) == 4;
+  // the right-hand side at N = 256, 512 and 1024 (FP32) stages its rows through
+  // shared memory
+  static constexpr bool X2S = (N == 256 || X2) && sizeof(T) == 4;
   template <int MODE> static void xpass_plain(const PassArgs& a) {
     if constexpr (XROW) {
       (void)a;
@@ -1177,31 +1181,11 @@ template <typename T, int N> struct Passes {
     if constexpr (X2S) {
       if (mode == XMODE_RHS) return xpass_staged<XMODE_RHS>(a);
       if (mode == XMODE_CONVECTIVE) return xpass_staged<XMODE_CONVECTIVE>(a);
-    }
-    if (mode == XMODE_CONVECTIVE) return xpass_plain<XMODE_CONVECTIVE>(a);
-    if constexpr (XROW) {
-      (void)a;
-      (void)mode;
-    } else if constexpr (X2) {
-      const size_t sm2 = X2Cfg<T, N>::SMEM;
-      if (mode == XMODE_STATS) {
-        prep(k_xpass2<T, N, XMODE_STATS>, sm2);
-        k_xpass2<T, N, XMODE_STATS><<<xgrid(), 128, sm2, a.st>>>(a);
-      } else {
-        prep(k_xpass2<T, N, XMODE_RHS>, sm2);
-        k_xpass2<T, N, XMODE_RHS><<<xgrid(), 128, sm2, a.st>>>(a);
-      }
     } else {
-      const size_t sm = XCfg<T, N>::SMEM;
-      dim3 block(32 * XCfg<T, N>::WARPS);
-      if (mode == XMODE_STATS) {
-        prep(k_xpass<T, N, XMODE_STATS>, sm);
-        k_xpass<T, N, XMODE_STATS><<<xgrid(), block, sm, a.st>>>(a);
-      } else {
-        prep(k_xpass<T, N, XMODE_RHS>, sm);
-        k_xpass<T, N, XMODE_RHS><<<xgrid(), block, sm, a.st>>>(a);
-      }
+      if (mode == XMODE_CONVECTIVE) return xpass_plain<XMODE_CONVECTIVE>(a);
     }
+    if (mode == XMODE_STATS) return xpass_plain<XMODE_STATS>(a);
+    if constexpr (!X2S) xpass_plain<XMODE_RHS>(a);
   }
   // The row X pass serves the right-hand side, the pressure inputs and the
   // statistics; the convective form needs the register X passes (it is
@@ -1270,15 +1254,13 @@ template <typename T, int N> struct PassesPS {
     if constexpr (MODE != XMODE_CONVECTIVE && (ROWS || B::XROW_OK)) {
       if (ROWS || a.xrow) return B::template xrow_launch<MODE, KS, SH>(a);
     }
-    if constexpr (B::X2) {
-      if constexpr (B::X2S && MODE == XMODE_RHS) {
-        // the right-hand side at N = 1024 stages its rows through shared memory
-        using SC = X2SCfg<T, N, KS>;
-        const long long rows = (long long)N * N / SC::ROWS;
-        const int grid = (int)(rows < B::sm_count() ? rows : B::sm_count());
-        go(k_xpass2s<T, N, KS, SH>, dim3(grid), dim3(SC::THREADS), SC::SMEM, a);
-        return;
-      }
+    if constexpr (B::X2S && MODE == XMODE_RHS) {
+      // the right-hand side at N = 256, 512 and 1024 stages its rows through shared memory
+      using SC = X2SCfg<T, N, KS>;
+      const long long rows = (long long)N * N / SC::ROWS;
+      const int grid = (int)(rows < B::sm_count() ? rows : B::sm_count());
+      go(k_xpass2s<T, N, KS, SH>, dim3(grid), dim3(SC::THREADS), SC::SMEM, a);
+    } else if constexpr (B::X2) {
       go(k_xpass2<T, N, MODE, KS, SH>, dim3(B::xgrid()), dim3(128), X2Cfg<T, N>::SMEM, a);
     } else if constexpr (!ROWS) {
       go(k_xpass<T, N, MODE, KS, SH>, dim3(B::xgrid()), dim3(32 * XCfg<T, N>::WARPS), XCfg<T, N>::SMEM, a);

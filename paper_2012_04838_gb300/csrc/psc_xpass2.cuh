@@ -1,4 +1,4 @@
-// X pass for N = 16 * 16 * G (G = 2: N = 512, G = 4: N = 1024).
+// X pass for N = 16 * 16 * G (G = 1: N = 256, G = 2: N = 512, G = 4: N = 1024).
 //
 // One row of N points is transformed by TH = 16 G threads holding 16 values
 // each.  With n = a + 16 b + 256 c and k = k0 + G k1 + 16 G k2
@@ -39,7 +39,7 @@ template <typename T, int N> struct X2Cfg {
   static constexpr size_t TW_BYTES = (size_t)(2 * 16 * TH + 16 * G) * sizeof(C);
   static constexpr size_t SMEM = LINE_BYTES * ROWS + ACC_BYTES + TW_BYTES;
   static constexpr int K = (N - 1) / 3;
-  static_assert(N == 512 || N == 1024, "X2 layout covers N = 512 and 1024");
+  static_assert(N == 256 || N == 512 || N == 1024, "X2 layout covers N = 256, 512 and 1024");
 };
 
 // Positions j + TH m (j < TH) of a length-N line split into 16 slots of TH,
@@ -49,9 +49,9 @@ __host__ __device__ constexpr int band_of_k(int N, int TH, int m, int K) {
   return (TH * m + TH - 1 <= K || TH * m >= N - K) ? 1 : (TH * m > K && TH * m + TH - 1 < N - K) ? 0 : 2;
 }
 
-// barrier over the TH threads of one row
+// barrier over the TH threads of one row (a warp holds two rows where TH = 16)
 template <int TH> __device__ __forceinline__ void row_sync(int id) {
-  if constexpr (TH == 32) {
+  if constexpr (TH <= 32) {
     __syncwarp();
   } else {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(TH) : "memory");
@@ -86,7 +86,10 @@ __device__ __forceinline__ void lane_dft(typename CT<T>::type (&v)[16], int r) {
       for (int i = 0; i < 16; ++i) v[i] = DIR < 0 ? mk(v[i].y, -v[i].x) : mk(-v[i].y, v[i].x);
     }
   };
-  if constexpr (G == 2) {
+  if constexpr (G == 1) {
+    (void)bfly;
+    (void)quarter;
+  } else if constexpr (G == 2) {
     bfly(1, r & 1);
   } else if constexpr (DIR < 0) {
     bfly(2, r & 2);
@@ -102,7 +105,7 @@ __device__ __forceinline__ void lane_dft(typename CT<T>::type (&v)[16], int r) {
 // The first DFT-16 of an inverse transform: slots m whose 16 G positions all
 // lie in the zero band for every thread (band_of_k == 0) are known zeros, and
 // the pruned codelet DftZ<16, +1, Z0, Z1> skips them (the generator emits it
-// for slots 6..9, the band of the 2/3 rule at N = 512 and 1024); a plain
+// for slots 6..9, the band of the 2/3 rule at N = 256, 512 and 1024); a plain
 // DFT-16 otherwise.  Adding a known zero is left out, so the sums are the same.
 template <int N, int KK> struct x2_first_inverse {
   static constexpr int TH = X2Cfg<float, N>::TH;
@@ -355,8 +358,8 @@ __device__ __forceinline__ bool x2_rhs_row(const YF& Y, const HA& after_a, const
 #pragma unroll
   for (int b = 0; b < 16; ++b) {
     const T w1 = W[b], w2 = z[b].x, w3 = z[b].y;
-    z[b] = mk((u2[b] * w3 - u3[b] * w2) * s2, (u3[b] * w1 - u1[b] * w3) * s2);  // (NL1, NL2)
-    W[b] = u1[b] * w2 - u2[b] * w1;                                              // NL3
+    z[b] = mk(det2(u2[b], w3, u3[b], w2) * s2, det2(u3[b], w1, u1[b], w3) * s2);  // (NL1, NL2)
+    W[b] = det2(u1[b], w2, u2[b], w1);                                            // NL3
   }
   x2fwd<T, N, KK, SHIFT>(z,
               [&](int kx, C X1, C X2) {
@@ -382,12 +385,12 @@ __device__ __forceinline__ bool x2_rhs_row(const YF& Y, const HA& after_a, const
   x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); },
                      z, ex, q, scale, phase);
 #pragma unroll
-  for (int b = 0; b < 16; ++b) u1[b] = u1[b] * z[b].x + u2[b] * z[b].y;
+  for (int b = 0; b < 16; ++b) u1[b] = dot2(u1[b], z[b].x, u2[b], z[b].y);
   // (dphi/dx3, 0)
   x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, q, scale, phase);
   after_b();
 #pragma unroll
-  for (int b = 0; b < 16; ++b) z[b] = mk(W[b] * s2, (u1[b] + u3[b] * z[b].x) * s2);  // (NL3, u.grad phi)
+  for (int b = 0; b < 16; ++b) z[b] = mk(W[b] * s2, fma(u3[b], z[b].x, u1[b]) * s2);  // (NL3, u.grad phi)
   x2fwd<T, N, KK, SHIFT>(z,
               [&](int kx, C X1, C X2) {
                 const long long i0 = 2 * ys + line * MP + kx;
@@ -634,14 +637,18 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : PSC_X2_MINB) k_xpass
 }
 
 // ---------------------------------------------------------------------------
-// Staged x pass (right-hand side, rotational or convective form; FP32,
-// N = 1024).  One CTA per SM holds X2SCfg::ROWS rows in flight; the input
-// streams of each row are copied into shared memory by bulk asynchronous
-// copies (TMA engine) one row ahead, in two groups completed on two mbarriers:
+// Staged x pass (right-hand side, rotational or convective form; FP32, N = 256,
+// 512 and 1024).  One CTA per SM holds X2SCfg::UNITS units in flight, a unit
+// being a row, or the two adjacent rows of a warp at N = 256; the input streams
+// of each unit are copied into shared memory by bulk asynchronous copies (TMA
+// engine) one unit ahead, in two groups completed on two mbarriers:
 // group A, the streams of the first inverse transforms, and group B, those of
-// the last ones (X2SGroups).  Each group of the next row is issued as soon as
-// the current row stops reading it, so global latency overlaps several
-// transforms, and the transforms read their inputs from shared memory.
+// the last ones (X2SGroups).  Each group of the next unit is issued as soon as
+// the current one stops reading it, so global latency overlaps several
+// transforms, and the transforms read their inputs from shared memory: a packed
+// transform reads every value twice (at p and N - p) and three streams serve
+// two transforms, 2.4 reads of each value, which at N = 256 left the unstaged
+// pass waiting for the L1 and L2 caches (62% of issue slots unused).
 // ---------------------------------------------------------------------------
 // Streams a staged row reads, as bit masks over the y-stage streams (a
 // stream's shared-memory slot is its index)
@@ -666,28 +673,38 @@ template <typename T, int N, int KK = (N - 1) / 3, int MODE = XMODE_RHS> struct 
   using C = typename CT<T>::type;
   using XC = X2Cfg<T, N>;
   using G = X2SGroups<MODE>;
-#ifndef PSC_X2S_ROWS
-#define PSC_X2S_ROWS 6
-#endif
   static constexpr int MP = row_pitch(KK + 1);
   static constexpr unsigned ROW_BYTES = (unsigned)(MP * sizeof(C));
-  static constexpr size_t STAGE_BYTES = (size_t)G::SLOTS * ROW_BYTES;
-  static constexpr size_t GROUP_BYTES = STAGE_BYTES + XC::LINE_BYTES;
-  // rows in flight: PSC_X2S_ROWS, fewer where longer rows (more streams, or the
-  // phase-shift sphere's cube) would not fit shared memory
-  static constexpr int rows_fit() {
-    int r = PSC_X2S_ROWS;
+  // a unit: the threads that wait for one set of copies (a whole number of warps)
+  static constexpr int RPU = XC::TH < 32 ? 32 / XC::TH : 1;  // rows per unit
+  static constexpr int UTH = XC::TH * RPU;                   // threads per unit
+  static constexpr unsigned UNIT_BYTES = ROW_BYTES * RPU;    // one stream of a unit
+  static constexpr size_t STAGE_BYTES = (size_t)G::SLOTS * UNIT_BYTES;
+  static constexpr size_t GROUP_BYTES = STAGE_BYTES + XC::LINE_BYTES * RPU;
+  // units in flight: 12 warps, what 168 registers a thread leave room for, fewer
+  // where longer rows (more streams, or the phase-shift sphere's cube) would not
+  // fit shared memory
+  static constexpr int units_fit() {
+    int r = 12 * 32 / UTH;
     while (r > 1 && GROUP_BYTES * r + XC::TW_BYTES + 2 * r * 8 > 227 * 1024) --r;
     return r;
   }
-  static constexpr int ROWS = rows_fit();
-  static constexpr int THREADS = XC::TH * ROWS;
-  static constexpr size_t TW_OFF = GROUP_BYTES * ROWS;
+  static constexpr int UNITS = units_fit();
+  static constexpr int ROWS = UNITS * RPU;
+  static constexpr int THREADS = UTH * UNITS;
+  static constexpr size_t TW_OFF = GROUP_BYTES * UNITS;
   static constexpr size_t BAR_OFF = TW_OFF + XC::TW_BYTES;
-  static constexpr size_t SMEM = BAR_OFF + 2 * ROWS * sizeof(unsigned long long);
+  static constexpr size_t SMEM = BAR_OFF + 2 * UNITS * sizeof(unsigned long long);
   static constexpr bool OK = ROW_BYTES % 16 == 0 && SMEM <= 227 * 1024;
   static_assert((G::A & G::B) == 0 && (G::A | G::B) < (1u << G::SLOTS), "stream groups are disjoint slots");
 };
+
+// AND of `pred` over a unit's UTH threads, which makes their earlier shared-memory
+// writes visible to one another
+template <int UTH> __device__ __forceinline__ bool unit_and(int id, bool pred) {
+  if constexpr (UTH == 32) return __all_sync(0xffffffffu, pred);
+  else return bar_and(id, UTH, pred);
+}
 
 template <typename T, int N, int KK = (N - 1) / 3, bool SHIFT = false, int MODE = XMODE_RHS>
 __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(PassArgs a) {
@@ -697,23 +714,24 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
   using G = typename SC::G;
   static_assert(SC::OK, "staged x pass: rows must be 16-byte multiples and fit shared memory");
   static_assert(MODE == XMODE_RHS || MODE == XMODE_CONVECTIVE, "staged x pass: right-hand side only");
-  constexpr int TH = XC::TH, G_ = XC::G, ROWS = SC::ROWS, MP = SC::MP;
+  constexpr int TH = XC::TH, G_ = XC::G, MP = SC::MP, RPU = SC::RPU, UTH = SC::UTH, UNITS = SC::UNITS;
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int lid = threadIdx.x / TH;
+  const int uid = threadIdx.x / UTH, sub = threadIdx.x % UTH / TH;  // unit, and row within it
   X2Roles<C> q;
   q.tid = threadIdx.x % TH;
   q.ra = q.tid / G_;
   q.rr = q.tid % G_;
   q.rk0 = bitrev_lane<G_>(q.rr);
-  q.bar = 1 + lid;
-  unsigned char* grp = smraw + (size_t)lid * SC::GROUP_BYTES;
-  C* stg = reinterpret_cast<C*>(grp);
-  C* ex = reinterpret_cast<C*>(grp + SC::STAGE_BYTES);
-  unsigned long long* barA = reinterpret_cast<unsigned long long*>(smraw + SC::BAR_OFF) + 2 * lid;
+  q.bar = 1 + uid;
+  unsigned char* grp = smraw + (size_t)uid * SC::GROUP_BYTES;
+  C* stg = reinterpret_cast<C*>(grp);  // [stream][row of the unit][MP]
+  C* ex = reinterpret_cast<C*>(grp + SC::STAGE_BYTES + (size_t)sub * XC::LINE_BYTES);
+  unsigned long long* barA = reinterpret_cast<unsigned long long*>(smraw + SC::BAR_OFF) + 2 * uid;
   unsigned long long* barB = barA + 1;
   const C* __restrict__ yb = static_cast<const C*>(a.yb);
   C* __restrict__ xb = static_cast<C*>(a.xb);
-  if (q.tid == 0) {
+  const bool leader = threadIdx.x % UTH == 0;
+  if (leader) {
     mbar_init(barA, 1);
     mbar_init(barB, 1);
     mbar_init_fence();
@@ -721,57 +739,62 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
   x2_twiddles<T, N>(reinterpret_cast<C*>(smraw + SC::TW_OFF), static_cast<const C*>(a.tw), q);
   const long long ys = a.d.ys;  // N*N*MP for a pass over the box
   const long long nlines = ys / MP;
-  const long long stride = (long long)gridDim.x * ROWS;
+  const long long stride = (long long)gridDim.x * SC::ROWS;
   const T scale = T(1.0 / ((double)N * N * N));
-  const bool leader = q.tid == 0;
   // bound of the waits; the failure-path test asks one more transaction byte
   // than the copies bring for the first row of CTA 0's first row group, so that
-  // row's wait runs out (every copy still lands)
+  // unit's wait runs out (every copy still lands)
   const unsigned long long lim = a.ctrl->wait_ns ? a.ctrl->wait_ns : 2000000000ull;
-  bool stall = a.ctrl->stall_test != 0 && blockIdx.x == 0 && lid == 0;
-  // copies of the streams in `mask` of row ln into their staging slots (one thread)
+  bool stall = a.ctrl->stall_test != 0 && blockIdx.x == 0 && uid == 0;
+  // copies of the streams in `mask` of the unit that starts at row ln into their
+  // staging slots (one thread; a unit's rows are adjacent in every stream)
   auto issue = [&](long long ln, unsigned mask, unsigned long long* bar) {
     fence_proxy_async_smem();
-    mbar_expect_tx(bar, (unsigned)__popc(mask) * SC::ROW_BYTES + (stall ? 16u : 0u));
+    mbar_expect_tx(bar, (unsigned)__popc(mask) * SC::UNIT_BYTES + (stall ? 16u : 0u));
     stall = false;
 #pragma unroll
     for (int st = 0; st < G::SLOTS; ++st) {
       if (!((mask >> st) & 1u)) continue;
       const long long src = st * ys + ln * MP;
-      if (PSC_OK_INDEX(src + MP - 1, (long long)Y_NSTREAM * ys, a.ctrl))
-        bulk_copy_g2s(stg + st * MP, yb + src, SC::ROW_BYTES, bar);
+      if (PSC_OK_INDEX(src + RPU * MP - 1, (long long)Y_NSTREAM * ys, a.ctrl))
+        bulk_copy_g2s(stg + st * RPU * MP, yb + src, SC::UNIT_BYTES, bar);
     }
   };
   T um = T(0);
   unsigned pa = 0, pb = 0;        // parity of the next phase to wait for
   bool ia = false, ib = false;    // a group issued and not yet waited for
   bool ok = true;
-  long long line = (long long)blockIdx.x * ROWS + lid;
+  long long line = ((long long)blockIdx.x * UNITS + uid) * RPU;  // first row of the unit
   if (line < nlines) {
     if (leader) {
       issue(line, G::A, barA);
       issue(line, G::B, barB);
     }
+    __syncwarp();
     ia = ib = true;
   }
 #pragma unroll 1
   for (; line < nlines; line += stride) {
     const long long next = line + stride;
-    // the row's first thread polls; the row barrier shares the outcome and
-    // makes the staged streams visible to the row's threads
-    ok = bar_and(q.bar, TH, leader ? mbar_wait(barA, pa, &a.ctrl->err, lim) : true);
+    // the unit's barrier shares the outcome of the wait and makes the staged
+    // streams visible to its threads.  Units of two warps: one thread polls
+    // (1024^3: 14.7 ms a launch, 14.8 with all).  Units of one warp: every lane
+    // does, because with one lane polling the warp stayed split afterwards and
+    // ran the row twice, that lane and the other 31 (256^3: 326 us against 165)
+    ok = unit_and<UTH>(q.bar, leader || UTH == 32 ? mbar_wait(barA, pa, &a.ctrl->err, lim) : true);
     if (!ok) break;
     pa ^= 1u;
     ia = false;
-    auto Y = [&](int st, int kx) -> C { return stg[st * MP + kx]; };
+    auto Y = [&](int st, int kx) -> C { return stg[(st * RPU + sub) * MP + kx]; };
     auto after_a = [&] {
       if (next < nlines) {
         if (leader) issue(next, G::A, barA);
+        if constexpr (UTH == 32) __syncwarp();
         ia = true;
       }
     };
     auto wait_b = [&] {
-      const bool w = bar_and(q.bar, TH, leader ? mbar_wait(barB, pb, &a.ctrl->err, lim) : true);
+      const bool w = unit_and<UTH>(q.bar, leader || UTH == 32 ? mbar_wait(barB, pb, &a.ctrl->err, lim) : true);
       if (w) {
         pb ^= 1u;
         ib = false;
@@ -781,14 +804,15 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
     auto after_b = [&] {
       if (next < nlines) {
         if (leader) issue(next, G::B, barB);
+        if constexpr (UTH == 32) __syncwarp();
         ib = true;
       }
     };
     if constexpr (MODE == XMODE_RHS)
-      ok = x2_rhs_row<T, N, false, KK, SHIFT>(Y, after_a, wait_b, after_b, xb, line, ys, ex, q, scale,
+      ok = x2_rhs_row<T, N, false, KK, SHIFT>(Y, after_a, wait_b, after_b, xb, line + sub, ys, ex, q, scale,
                                               a.want_umax != 0, um, a.ctrl, a.phase);
     else
-      ok = x2_conv_row<T, N, KK, SHIFT>(Y, after_a, wait_b, after_b, xb, line, ys, ex, q, scale,
+      ok = x2_conv_row<T, N, KK, SHIFT>(Y, after_a, wait_b, after_b, xb, line + sub, ys, ex, q, scale,
                                         a.want_umax != 0, um, a.ctrl, a.phase);
     if (!ok) break;
   }
