@@ -657,7 +657,7 @@ psc_status do_init(psc_sim* s) {
   const double n3 = (double)d.N * d.N * d.N;
   launch(s, PSC_K_OTHER, 4, [&] {
     k_ic_draw<<<blocks, 256, 0, s->st>>>(d, (unsigned long long)s->p.seed, z);
-    k_shells<double><<<s->nshell, 256, 0, s->st>>>(d, z, nullptr, s->nshell, shells);
+    k_shells<double><<<s->nshell * SHELL_PARTS, 256, 0, s->st>>>(d, z, nullptr, s->nshell, shells);
     k_ic_factors<<<1, 32, 0, s->st>>>(s->nshell, shells, 1.0 / (2.0 * n3 * n3), K0, shape, s->p.kF, fac);
     k_ic_finish<T><<<blocks, 256, 0, s->st>>>(d, z, fac, tg ? 1 : 0, s->ws + s->L.U);
   });
@@ -688,8 +688,8 @@ psc_status do_stats(psc_sim* s, double* Ek, double* Ephi, int cap, int* nshell, 
   });
   double* shells = (double*)(s->ws + s->L.shells);
   launch(s, PSC_K_OTHER, 2, [&] {
-    k_reduce_moments<<<1, NQ * REDUCE_LANES, 0, s->st>>>(a.partials, s->tb->xwarps, s->ctrl);
-    k_shells<T><<<s->nshell, 256, 0, s->st>>>(d, U, (const unsigned char*)U + 3 * d.S * (s->fp64 ? 16 : 8),
+    k_reduce_moments<<<NQ, 256, 0, s->st>>>(a.partials, s->tb->xwarps, s->ctrl);
+    k_shells<T><<<s->nshell * SHELL_PARTS, 256, 0, s->st>>>(d, U, (const unsigned char*)U + 3 * d.S * (s->fp64 ? 16 : 8),
                                                s->nshell, shells);
   });
   PSC_LAUNCHED("psc_spectra_and_stats");

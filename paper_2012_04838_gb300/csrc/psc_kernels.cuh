@@ -4,6 +4,8 @@
 // Kernels that are not templates are static: several units compile this header.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include "psc_scalars.cuh"
 
 namespace psc {
@@ -196,46 +198,38 @@ __global__ void k_iftab(int K, const Ctrl* ctrl, double nu, double D, T* eu, T* 
   b_iftab<T>(K, ctrl, nu, D, eu, ep, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-// Fixed-order block sum of one double (every thread passes its value; the
-// result is valid in thread 0).
-__device__ __forceinline__ double block_sum(double v, double* sm) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) sm[wid] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sm[w];
-  return s;
-}
-
-// floor(sqrt(a)) for 0 <= a < 2^46: an FP32 estimate corrected in integers
+// floor(sqrt(a)) for 0 <= a < 2^30: an FP32 estimate corrected in integers
 // (exact; the FP64 square root is slow on this part)
-__device__ __forceinline__ long long isqrt_floor(long long a) {
+__device__ __forceinline__ int isqrt_floor(int a) {
   if (a <= 0) return 0;
-  long long s = (long long)sqrtf((float)a);
+  int s = (int)sqrtf((float)a);
   while (s * s > a) --s;
   while ((s + 1) * (s + 1) <= a) ++s;
   return s;
 }
 
-// Shell n = floor(|k| + 1/2), i.e. n^2 - n < |k|^2 <= n^2 + n.  One CTA per
-// shell sums w |u|^2, w |phi|^2, |k|^2 w |u|^2, |k|^2 w |phi|^2 and
-// w Re(conj(phi) u2) over the shell's stored modes (w = 1 at kx = 0, else 2).
-// Each thread accumulates in the state's precision (compensated sums in FP32,
-// since FP64 arithmetic is slow on this part), then the CTA adds the threads'
-// sums in FP64 in a fixed order.  out[q * nshell + n] holds the raw sums.
+// Shell n = floor(|k| + 1/2), i.e. n^2 - n < |k|^2 <= n^2 + n.  A cluster of
+// SHELL_PARTS CTAs per shell sums w |u|^2, w |phi|^2, |k|^2 w |u|^2, |k|^2 w |phi|^2
+// and w Re(conj(phi) u2) over the shell's stored modes (w = 1 at kx = 0, else
+// 2), each CTA over its share of the (kz, ky) columns.  Each thread accumulates
+// in the state's precision (compensated sums in FP32, since FP64 arithmetic is
+// slow on this part), then the threads' and the CTAs' sums are added in FP64 in
+// a fixed order, the CTAs' through distributed shared memory.
+// out[q * nshell + n] holds the raw sums.  The loads of a column are short runs
+// scattered over the state, so the pass is bound by their latency: one CTA per
+// shell left most of the chip idle (115 us at 128^3, 1377 us at 512^3).
+constexpr int SHELL_PARTS = 8;
 template <typename T>
-__global__ void __launch_bounds__(256) k_shells(Dims d, const void* u_, const void* phi_, int nshell,
-                                               double* out) {
+__global__ void __cluster_dims__(SHELL_PARTS, 1, 1) __launch_bounds__(256)
+k_shells(Dims d, const void* u_, const void* phi_, int nshell, double* out) {
   using C = typename CT<T>::type;
-  __shared__ double sm[32];
-  const C* u = static_cast<const C*>(u_);
-  const C* phi = static_cast<const C*>(phi_);
-  const int n = blockIdx.x;
-  const long long lo = n == 0 ? -1 : (long long)n * n - n;  // exclusive
-  const long long hi = n == 0 ? 0 : (long long)n * n + n;   // inclusive
+  __shared__ double warp_sums[8][NSQ];
+  __shared__ double cta_sums[NSQ];
+  const C* __restrict__ u = static_cast<const C*>(u_);
+  const C* __restrict__ phi = static_cast<const C*>(phi_);
+  const int n = blockIdx.x / SHELL_PARTS, part = blockIdx.x % SHELL_PARTS;
+  const int lo = n == 0 ? -1 : n * n - n;  // exclusive
+  const int hi = n == 0 ? 0 : n * n + n;   // inclusive; |k|^2 < 2^24
   const int kb = (n + 1) < d.K ? (n + 1) : d.K;
   const int side = 2 * kb + 1;
   MomentSum<T> acc[NSQ];
@@ -243,15 +237,15 @@ __global__ void __launch_bounds__(256) k_shells(Dims d, const void* u_, const vo
   // range limits); the raw sums are restored in FP64 at the end
   const double n3 = (double)d.N * d.N * d.N;
   const T sc = (T)(1.0 / n3);
-  for (int q = threadIdx.x; q < side * side; q += blockDim.x) {
+  for (int q = part * blockDim.x + threadIdx.x; q < side * side; q += SHELL_PARTS * blockDim.x) {
     const int kz = q / side - kb, ky = q % side - kb;
-    const long long r2 = (long long)kz * kz + (long long)ky * ky;
+    const int r2 = kz * kz + ky * ky;
     if (r2 > hi) continue;
-    const long long x0 = (lo - r2 < 0) ? 0 : isqrt_floor(lo - r2) + 1;
-    long long x1 = isqrt_floor(hi - r2);
+    const int x0 = (lo - r2 < 0) ? 0 : isqrt_floor(lo - r2) + 1;
+    int x1 = isqrt_floor(hi - r2);
     if (x1 > d.K) x1 = d.K;
     const long long base = ((long long)(kz + d.K) * d.P + (ky + d.K)) * d.M;
-    for (long long kx = x0; kx <= x1; ++kx) {
+    for (int kx = x0; kx <= x1; ++kx) {
       const long long i = base + kx;
       const T w = kx == 0 ? T(1) : T(2);
       const T k2 = (T)(r2 + kx * kx);  // exact: |k|^2 < 2^24
@@ -268,30 +262,45 @@ __global__ void __launch_bounds__(256) k_shells(Dims d, const void* u_, const vo
       }
     }
   }
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
   for (int q = 0; q < NSQ; ++q) {
-    const double s = block_sum(acc[q].value(), sm);
-    if (threadIdx.x == 0) out[q * nshell + n] = s * n3 * n3;
-    __syncthreads();
+    double v = acc[q].value();
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) warp_sums[wid][q] = v;
   }
+  __syncthreads();
+  if (threadIdx.x < NSQ) {
+    double s = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += warp_sums[w][threadIdx.x];
+    cta_sums[threadIdx.x] = s;
+  }
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  cl.sync();
+  if (part == 0 && threadIdx.x < NSQ) {
+    double s = 0.0;
+    for (int r = 0; r < SHELL_PARTS; ++r) s += *cl.map_shared_rank(&cta_sums[threadIdx.x], r);
+    out[threadIdx.x * nshell + n] = s * n3 * n3;
+  }
+  cl.sync();  // a CTA's shared memory stays until the first one has read it
 }
 
 #ifndef PSC_SHELLS_ONLY
-// Sum the X-pass partials over their nw rows in a fixed order: 32 threads per
-// moment, each over every 32nd row (consecutive threads read consecutive
-// values, and the loads of a thread are independent of its sum), then one
-// thread per moment over the 32 sums.
-constexpr int REDUCE_LANES = 32;
-static __global__ void __launch_bounds__(NQ * REDUCE_LANES) k_reduce_moments(const double* partials, int nw,
-                                                                             Ctrl* ctrl) {
-  __shared__ double sm[NQ * REDUCE_LANES];
-  const int q = threadIdx.x % NQ, l = threadIdx.x / NQ;
+// Sum the X-pass partials over their nw rows in a fixed order: one CTA per
+// moment, each thread over every 256th row (independent loads in flight), then
+// the threads' sums.  768 threads of one CTA took 72 us over the 9728 rows of
+// 512^3, one thread per moment 0.7 ms; this 12 us.
+static __global__ void __launch_bounds__(256) k_reduce_moments(const double* partials, int nw, Ctrl* ctrl) {
+  __shared__ double sm[8];
+  const int q = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double s = 0.0;
-#pragma unroll 8
-  for (int w = l; w < nw; w += REDUCE_LANES) s += partials[(long long)w * NQ + q];
-  sm[threadIdx.x] = s;
+#pragma unroll 4
+  for (int w = threadIdx.x; w < nw; w += 256) s += partials[(long long)w * NQ + q];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (lane == 0) sm[wid] = s;
   __syncthreads();
-  if (l != 0) return;
-  for (int i = 1; i < REDUCE_LANES; ++i) s += sm[i * NQ + q];
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < 8; ++w) s += sm[w];
   ctrl->moments[q] = s;
 }
 
@@ -383,7 +392,7 @@ __global__ void k_ic_finish(Dims d, const double2* z, const double* fac, int tay
   int kx, ky, kz;
   mode_of(d, i, kx, ky, kz);
   const long long k2 = (long long)kx * kx + (long long)ky * ky + (long long)kz * kz;
-  long long n = isqrt_floor(k2);
+  int n = isqrt_floor((int)k2);
   if (k2 > n * n + n) ++n;
   const double f = outside_sphere(d, k2) ? 0.0 : fac[n];
   double v[3][2];

@@ -134,9 +134,9 @@ extern "C" psc_status psc_shell_spectra_noalloc(const void* state, int32_t N, in
   // so nothing left from an earlier call is read
   const unsigned char* u = static_cast<const unsigned char*>(state);
   if (precision == PSC_FP64)
-    psc::k_shells<double><<<nshell, 256, 0, st>>>(d, u, u + 3 * d.S * 16, nshell, scratch);
+    psc::k_shells<double><<<nshell * psc::SHELL_PARTS, 256, 0, st>>>(d, u, u + 3 * d.S * 16, nshell, scratch);
   else
-    psc::k_shells<float><<<nshell, 256, 0, st>>>(d, u, u + 3 * d.S * 8, nshell, scratch);
+    psc::k_shells<float><<<nshell * psc::SHELL_PARTS, 256, 0, st>>>(d, u, u + 3 * d.S * 8, nshell, scratch);
   const double n3 = (double)N * N * N;
   k_noalloc_finish<<<(nshell + 127) / 128, 128, 0, st>>>(scratch, nshell, 1.0 / (2.0 * n3 * n3), Ek, Ephi);
   e = cudaGetLastError();

@@ -812,39 +812,45 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
       xfwd<T, N, KK, SHIFT>(z, store(2), ex, tw, t, a.phase);
     } else {
       // statistics: moments of the diagonal velocity gradients and the scalar
-      // gradient (Eqs. 11-12), |omega|^2, u.u, phi u2, phi^2 (Eq. 13)
-      T s13[J2][R2];
-      auto mom = [&](int q, T v) { (void)q; return v; };
-      (void)mom;
-      auto acc234 = [&](int q, int j, int k2, T v) {
-        const T v2 = v * v;
-        acc[q].add(v2);
-        acc[q + 1].add(v2 * v);
-        acc[q + 2].add(v2 * v2);
-        (void)j; (void)k2;
+      // gradient (Eqs. 11-12), |omega|^2, u.u, phi u2, phi^2 (Eq. 13).  The
+      // thread's points of one field are added up first, in four short chains,
+      // and join the compensated sum once per field and row: a compensated add
+      // per point is four dependent operations for each of 20 sums (the pass
+      // took 108 us at 128^3 against 38 us for the right-hand side).
+      constexpr int NP = J2 * R2;
+      T s13[NP], f1[NP], f2[NP];
+      auto split = [&]() {
+#pragma unroll
+        for (int j = 0; j < J2; ++j)
+#pragma unroll
+          for (int k2 = 0; k2 < R2; ++k2) { f1[j * R2 + k2] = z[j][k2].x; f2[j * R2 + k2] = z[j][k2].y; }
+      };
+      // acc[q] += sum over the points of term(i)
+      auto put = [&](int q, auto&& term) {
+        T s[4] = {T(0), T(0), T(0), T(0)};
+#pragma unroll
+        for (int i = 0; i < NP; ++i) s[i & 3] += term(i);
+        acc[q].add((s[0] + s[1]) + (s[2] + s[3]));
+      };
+      auto mom3 = [&](int q, const T (&f)[NP]) {
+        put(q, [&](int i) { return f[i] * f[i]; });
+        put(q + 1, [&](int i) { return f[i] * f[i] * f[i]; });
+        put(q + 2, [&](int i) { return (f[i] * f[i]) * (f[i] * f[i]); });
       };
       // (u1, u3)
       xinv<T, N, true, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UZ, kx); }, z, ex, tw, t, scale, a.phase);
+      split();
+      put(0, [&](int i) { return f1[i] * f1[i] + f2[i] * f2[i]; });
 #pragma unroll
-      for (int j = 0; j < J2; ++j)
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) {
-          const T u1 = z[j][k2].x, u3 = z[j][k2].y;
-          acc[0].add(u1 * u1 + u3 * u3);
-          s13[j][k2] = fabs(u1) + fabs(u3);
-        }
+      for (int i = 0; i < NP; ++i) s13[i] = fabs(f1[i]) + fabs(f2[i]);
       // (u2, phi)
       xinv<T, N, true, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UY, kx); x2 = Y(Y_PHI, kx); }, z, ex, tw, t, scale, a.phase);
+      split();
+      put(0, [&](int i) { return f1[i] * f1[i]; });
+      put(20, [&](int i) { return f2[i] * f1[i]; });
+      put(21, [&](int i) { return f2[i] * f2[i]; });
 #pragma unroll
-      for (int j = 0; j < J2; ++j)
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) {
-          const T u2 = z[j][k2].x, ph = z[j][k2].y;
-          acc[0].add(u2 * u2);
-          acc[20].add(ph * u2);
-          acc[21].add(ph * ph);
-          um = max_keep_nan(um, s13[j][k2] + fabs(u2));
-        }
+      for (int i = 0; i < NP; ++i) um = max_keep_nan(um, s13[i] + fabs(f1[i]));
       // (omega_1, omega_2)
       xinv<T, N, true, KK, SHIFT>(
           [&](int kx, C& x1, C& x2) {
@@ -852,11 +858,8 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
             x2 = csub(Y(Y_DZUX, kx), mul_ik(Y(Y_UZ, kx), T(kx)));
           },
           z, ex, tw, t, scale, a.phase);
-#pragma unroll
-      for (int j = 0; j < J2; ++j)
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2)
-          acc[1].add(z[j][k2].x * z[j][k2].x + z[j][k2].y * z[j][k2].y);
+      split();
+      put(1, [&](int i) { return f1[i] * f1[i] + f2[i] * f2[i]; });
       // (omega_3, dphi/dx1)
       xinv<T, N, true, KK, SHIFT>(
           [&](int kx, C& x1, C& x2) {
@@ -864,39 +867,25 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
             x2 = mul_ik(Y(Y_PHI, kx), T(kx));
           },
           z, ex, tw, t, scale, a.phase);
-#pragma unroll
-      for (int j = 0; j < J2; ++j)
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) {
-          acc[1].add(z[j][k2].x * z[j][k2].x);
-          acc234(11, j, k2, z[j][k2].y);
-        }
+      split();
+      put(1, [&](int i) { return f1[i] * f1[i]; });
+      mom3(11, f2);
       // (dphi/dx2, dphi/dx3)
       xinv<T, N, true, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DYPHI, kx); x2 = Y(Y_DZPHI, kx); }, z, ex, tw, t,
                  scale, a.phase);
-#pragma unroll
-      for (int j = 0; j < J2; ++j)
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) {
-          acc234(14, j, k2, z[j][k2].x);
-          acc234(17, j, k2, z[j][k2].y);
-        }
+      split();
+      mom3(14, f1);
+      mom3(17, f2);
       // (du1/dx1, du2/dx2)
       xinv<T, N, true, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_UX, kx), T(kx)); x2 = Y(Y_DYUY, kx); }, z,
                  ex, tw, t, scale, a.phase);
-#pragma unroll
-      for (int j = 0; j < J2; ++j)
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) {
-          acc234(2, j, k2, z[j][k2].x);
-          acc234(5, j, k2, z[j][k2].y);
-        }
+      split();
+      mom3(2, f1);
+      mom3(5, f2);
       // (du3/dx3, 0)
       xinv<T, N, true, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZUZ, kx); x2 = zero; }, z, ex, tw, t, scale, a.phase);
-#pragma unroll
-      for (int j = 0; j < J2; ++j)
-#pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) acc234(8, j, k2, z[j][k2].x);
+      split();
+      mom3(8, f1);
     }
   }
 
