@@ -40,6 +40,12 @@ constexpr int kThreads = 128;
 enum { BP_FAMP = 0, BP_ZINV, BP_YINV, BP_XPASS, BP_CFL, BP_YFWD, BP_ZFWD, BP_COMBINE, BP_HOLD, BP_N };
 constexpr int kCombinePerThread = 4;  // compact modes per thread of a combine item
 constexpr int kXGroupsPerWarp = 2;    // row groups per warp of an X-pass item
+// Warps of a CTA that take rows in the X pass: two where the rows' velocities are
+// parked in shared memory (96^3 and 192^3, 65 KB with four), which would
+// otherwise hold every pass of the kernel to three CTAs per SM.
+template <int N> struct XItem {
+  static constexpr int WARPS = pp::XCfg<float, N>::STASH ? 2 : pp::XCfg<float, N>::WARPS;
+};
 
 struct Seg {
   long long start;  // index of the segment's first item within the stage
@@ -97,7 +103,7 @@ template <int N> int tiles_of(int pass, int stage, const PscBatchBox& b) {
     case BP_YINV: return gx * N;
     case BP_XPASS: {
       const long long groups = ((long long)N * N + XC::LPW - 1) / XC::LPW;
-      const long long per = (long long)XC::WARPS * kXGroupsPerWarp;
+      const long long per = (long long)XItem<N>::WARPS * kXGroupsPerWarp;
       return (int)((groups + per - 1) / per);
     }
     case BP_CFL: return (stage == 1 && b.cfl_on) ? 1 : 0;
@@ -125,7 +131,7 @@ inline int tiles_per_item(int pass) {
 
 template <int N> size_t smem_of() {
   constexpr int W = width_of<N>();
-  const size_t a = pp::StridedSmem<float, N, W>::BYTES, x = pp::XCfg<float, N>::SMEM;
+  const size_t a = pp::StridedSmem<float, N, W>::BYTES, x = pp::XCfg<float, N>::smem(XItem<N>::WARPS);
   return a > x ? a : x;
 }
 
@@ -194,7 +200,7 @@ __device__ __forceinline__ void run_item(const PscBatchBox& b, int pass, int til
       break;
     case BP_ZINV: b_zinv<float, N, false, W>(a, strided); break;
     case BP_YINV: b_yinv<float, N, YMODE_RHS, W>(a, strided); break;
-    case BP_XPASS: b_xpass<float, N, XMODE_RHS>(a, Tctx{tid, 0, tile, 0, kThreads, 1, ntiles, smem}); break;
+    case BP_XPASS: b_xpass<float, N, XMODE_RHS, (N - 1) / 3, false, XItem<N>::WARPS>(a, Tctx{tid, 0, tile, 0, kThreads, 1, ntiles, smem}); break;
     case BP_CFL:
       // dt for Eq. 10 from the maximum the X pass reduced, then the integrating
       // factors of that dt (K + 1 <= kThreads entries)
@@ -255,7 +261,9 @@ constexpr unsigned long long kWaitNs = 2000000000ull;
 constexpr unsigned long long kStallTestWaitNs = 50000000ull;
 
 #ifndef PSCB_MINB
-#define PSCB_MINB 3  // CTAs per SM the register budget is sized for
+// CTAs per SM the register budget is sized for (63 boxes, ms a step: 3 / 4 / 5 / 6
+// CTAs 8.24 / 7.44 / 7.86 / 7.93; more of them spill)
+#define PSCB_MINB 4
 #endif
 template <int STAGE, bool BIG>
 __global__ void __launch_bounds__(kThreads, PSCB_MINB)

@@ -445,7 +445,9 @@ template <typename T, int N> struct XCfg {
   // transposed forward plan (n2 < R1, k1 < R2), each stored [j][k1][t] so the
   // lanes of a row read consecutive entries
   static constexpr size_t TW_BYTES = (size_t)2 * N * sizeof(C);
-  static constexpr size_t SMEM = LINE_BYTES * LPW * WARPS + TW_BYTES;
+  // shared memory of a CTA in which `warps` warps take rows
+  __host__ __device__ static constexpr size_t smem(int warps) { return LINE_BYTES * LPW * warps + TW_BYTES; }
+  static constexpr size_t SMEM = smem(WARPS);
 };
 
 // Positions s0 .. s0 + w - 1 of a length-N axis truncated to |k| <= K: 1 if all
@@ -584,7 +586,8 @@ __device__ __forceinline__ void umax_update(Ctrl* c, double v) {
   atomicMax(&c->umax_bits, (unsigned long long)__double_as_longlong(v));
 }
 
-template <typename T, int N, int MODE, int KK = (N - 1) / 3, bool SHIFT = false>
+// XW: warps of the CTA that take rows (the others help with the tables only)
+template <typename T, int N, int MODE, int KK = (N - 1) / 3, bool SHIFT = false, int XW = XCfg<T, N>::WARPS>
 __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
   using C = typename CT<T>::type;
   using PL = PlanD<N>;
@@ -599,7 +602,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
   T* stash = reinterpret_cast<T*>(myline + XC::EXCH * sizeof(C));
   const C* PSC_RESTRICT yb = static_cast<const C*>(a.yb);
   C* PSC_RESTRICT xb = static_cast<C*>(a.xb);
-  C* tw = reinterpret_cast<C*>(smraw + XC::LINE_BYTES * LPW * XC::WARPS);
+  C* tw = reinterpret_cast<C*>(smraw + XC::LINE_BYTES * LPW * XW);
   {
     const C* PSC_RESTRICT twg = static_cast<const C*>(a.tw);
     for (int i = tcx.tx; i < N; i += tcx.bdx) {
@@ -626,8 +629,8 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
   MomentSum<T> acc[MODE == XMODE_STATS ? NQ : 1];
 
 #pragma unroll 1
-  for (long long grp = (long long)tcx.bx * XC::WARPS + wid; grp * LPW < nlines;
-       grp += (long long)tcx.gdx * XC::WARPS) {
+  for (long long grp = wid < XW ? (long long)tcx.bx * XW + wid : nlines; grp * LPW < nlines;
+       grp += (long long)tcx.gdx * XW) {
     const long long line = grp * LPW + g;
     const bool valid = FULL || line < nlines;
     const C* PSC_RESTRICT row = yb + line * MP;
@@ -898,7 +901,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
     if (lane == 0) umax_update(a.ctrl, umax);
   }
   if constexpr (MODE == XMODE_STATS) {
-    const long long gw = (long long)tcx.bx * XC::WARPS + wid;
+    const long long gw = (long long)tcx.bx * XW + wid;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       double v = acc[q].value();
@@ -917,11 +920,16 @@ template <typename T, int N, int MODE, bool SPHERE> constexpr int xpass_ctas() {
   if (XCfg<T, N>::PER <= 8) return MODE == XMODE_STATS ? 3 : 5;
   return MODE == XMODE_STATS || (MODE == XMODE_CONVECTIVE && SPHERE) ? 2 : 3;
 }
+// Warps per CTA: one where four would leave SMs without a CTA (32^3 has 128 warps
+// of rows: four to a CTA used 32 SMs, and FP64 is bound by the pipe of each)
+template <typename T, int N> struct XWarps {
+  static constexpr int value = N <= 48 ? 1 : XCfg<T, N>::WARPS;
+};
 template <typename T, int N, int MODE, int KK = (N - 1) / 3, bool SHIFT = false>
-__global__ void __launch_bounds__(32 * XCfg<T, N>::WARPS, xpass_ctas<T, N, MODE, (KK > (N - 1) / 3)>())
+__global__ void __launch_bounds__(32 * XWarps<T, N>::value, xpass_ctas<T, N, MODE, (KK > (N - 1) / 3)>())
 k_xpass(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  b_xpass<T, N, MODE, KK, SHIFT>(a, hw_ctx(smraw));
+  b_xpass<T, N, MODE, KK, SHIFT, XWarps<T, N>::value>(a, hw_ctx(smraw));
 }
 
 }  // namespace psc
@@ -952,6 +960,7 @@ template <typename T, int N> struct Passes {
   // at the sizes with the register X pass, for testing
   static constexpr bool XROW = !X2 && N / TPL > 64;
   static constexpr bool XROW_OK = !X2;
+  static constexpr int XW = XWarps<T, N>::value;  // warps per CTA of the register X pass
   using XRC = XRowCfg<T, N>;
   static int xrow_grid() {
     const long long g = ((long long)N * N + XRC::WR - 1) / XRC::WR;
@@ -961,7 +970,7 @@ template <typename T, int N> struct Passes {
   // X-pass CTAs (row X pass) or warps (register X passes) that write statistics partials
   static int xwarps() {
     if constexpr (XROW) return xrow_grid();
-    else return xgrid() * (X2 ? 4 : XCfg<T, N>::WARPS);
+    else return xgrid() * (X2 ? 4 : XW);
   }
   // grid: one CTA per statistics partials slot (xwarps()) except where the
   // row X pass is the only one
@@ -984,7 +993,7 @@ template <typename T, int N> struct Passes {
       return (int)(g < cap ? g : cap);
     } else {
       const long long groups = ((long long)N * N + XCfg<T, N>::LPW - 1) / XCfg<T, N>::LPW;
-      long long g = (groups + XCfg<T, N>::WARPS - 1) / XCfg<T, N>::WARPS;
+      long long g = (groups + XW - 1) / XW;
       const long long cap = 152 * 8;
       return (int)(g < cap ? g : cap);
     }
@@ -1151,9 +1160,9 @@ template <typename T, int N> struct Passes {
       prep(k_xpass2<T, N, MODE>, sm2);
       k_xpass2<T, N, MODE><<<xgrid(), 128, sm2, a.st>>>(a);
     } else {
-      const size_t sm = XCfg<T, N>::SMEM;
+      const size_t sm = XCfg<T, N>::smem(XW);
       prep(k_xpass<T, N, MODE>, sm);
-      k_xpass<T, N, MODE><<<xgrid(), dim3(32 * XCfg<T, N>::WARPS), sm, a.st>>>(a);
+      k_xpass<T, N, MODE><<<xgrid(), 32 * XW, sm, a.st>>>(a);
     }
   }
   // the staged x pass of the right-hand side (rotational or convective form)
@@ -1252,7 +1261,7 @@ template <typename T, int N> struct PassesPS {
     } else if constexpr (B::X2) {
       go(k_xpass2<T, N, MODE, KS, SH>, dim3(B::xgrid()), dim3(128), X2Cfg<T, N>::SMEM, a);
     } else if constexpr (!ROWS) {
-      go(k_xpass<T, N, MODE, KS, SH>, dim3(B::xgrid()), dim3(32 * XCfg<T, N>::WARPS), XCfg<T, N>::SMEM, a);
+      go(k_xpass<T, N, MODE, KS, SH>, dim3(B::xgrid()), dim3(32 * B::XW), XCfg<T, N>::smem(B::XW), a);
     }
   }
   // the 8-stream z-inverse serves the statistics (unshifted) and the
