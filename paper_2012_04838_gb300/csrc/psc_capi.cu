@@ -1,5 +1,6 @@
 // Host side of the C ABI (include/psc.h): parameter checks, workspace
 // layout, stage orchestration and assembly of the statistics record.
+#include <algorithm>
 #include <array>
 #include <cmath>
 #include <cstdio>
@@ -1115,21 +1116,52 @@ psc_status psc_batch_create(psc_sim* const* sims, int32_t n, void* stream, psc_b
     sims[i]->profiling = false;
     step0[i] = sims[i]->step;
     launch0[i] = sims[i]->launches;
-    sims[i]->share = n;
   }
+  // The members' steps as a graph: the largest first, each forked off as soon as
+  // the workspaces of the members under way leave room for its own within
+  // kBatchBytes (by a model of their run times: grid points and a constant), so
+  // that small boxes fill the chip together while what they stream stays near
+  // the L2 cache's size.  48 x 64^3 + 12 x 96^3 + 3 x 128^3, ms a step: all 63 at
+  // once 4.92; 20 / 60 / 110 / 180 / 240 / 400 / 1000 MB under way 8.92 / 5.84 /
+  // 4.82 / 4.61 / 4.37 / 4.35 / 4.59.
+  constexpr size_t kBatchBytes = (size_t)320 << 20;
+  std::vector<int> order(n);
+  for (int i = 0; i < n; ++i) order[i] = i;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return sims[x]->L.total > sims[y]->L.total; });
+  struct Running {
+    double end;
+    int i;
+  };
+  std::vector<Running> run;
+  size_t used = 0;
+  double clock = 0.0;
+  int last = -1;  // the member whose end made room last
   cudaError_t e = cudaStreamBeginCapture(b->st, cudaStreamCaptureModeRelaxed);
   psc_status st = PSC_OK;
   if (e == cudaSuccess) e = cudaEventRecord(b->events[0], b->st);
-  for (int i = 0; i < n && e == cudaSuccess && st == PSC_OK; ++i) {
+  for (int k = 0; k < n && e == cudaSuccess && st == PSC_OK; ++k) {
+    const int i = order[k];
     psc_sim* m = sims[i];
     if (m->st != b->st) e = cudaStreamWaitEvent(m->st, b->events[0], 0);
-    if (e != cudaSuccess) break;
-    st = m->fp64 ? do_step<double>(m, 1) : do_step<float>(m, 1);
-    if (st == PSC_OK && m->st != b->st) {
-      e = cudaEventRecord(b->events[i + 1], m->st);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(b->st, b->events[i + 1], 0);
+    while (!run.empty() && used + m->L.total > kBatchBytes && e == cudaSuccess) {
+      auto it = std::min_element(run.begin(), run.end(), [](const Running& x, const Running& y) { return x.end < y.end; });
+      clock = std::max(clock, it->end);
+      last = it->i;
+      used -= sims[last]->L.total;
+      run.erase(it);
+      e = cudaStreamWaitEvent(m->st, b->events[last + 1], 0);
     }
+    if (last >= 0 && e == cudaSuccess) e = cudaStreamWaitEvent(m->st, b->events[last + 1], 0);
+    if (e != cudaSuccess) break;
+    const double N = m->d.N;
+    used += m->L.total;
+    run.push_back(Running{clock + N * N * N + 3.0e5, i});
+    m->share = (int)std::max<size_t>(1, std::min<size_t>(n, kBatchBytes / m->L.total));
+    st = m->fp64 ? do_step<double>(m, 1) : do_step<float>(m, 1);
+    if (st == PSC_OK) e = cudaEventRecord(b->events[i + 1], m->st);
   }
+  for (int i = 0; i < n && e == cudaSuccess && st == PSC_OK; ++i)
+    if (sims[i]->st != b->st) e = cudaStreamWaitEvent(b->st, b->events[i + 1], 0);
   cudaGraph_t g = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(b->st, &g);
   for (int i = 0; i < n; ++i) {
