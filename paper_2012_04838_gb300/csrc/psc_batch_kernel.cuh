@@ -187,6 +187,7 @@ __device__ __forceinline__ void run_item(const PscBatchBox& b, int pass, int til
   a.shift = 0;
   a.xrow = 0;
   a.force.on = a.cfl.on = 0;
+  a.pdl = 0;
   a.share = 1;
   a.st = nullptr;
   const Tctx strided{tid % W, tid / W, tile % gx, tile / gx, W, LPL, gx, smem};

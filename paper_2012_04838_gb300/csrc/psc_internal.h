@@ -138,9 +138,29 @@ struct PassArgs {
   int xrow;         // 1: the shared-memory row X pass where the register one exists
   ForceArgs force;
   CflArgs cfl;
+  int pdl;          // 1: programmatic dependent launches (launch_kernel)
   int share;        // boxes whose passes run on the chip at the same time (at least 1)
   cudaStream_t st;
 };
+
+// Launch k on st.  pdl: as a programmatic dependent of the kernel before it in
+// the stream (every kernel launched so calls pdl_wait()).  Which grids: pdl_pays()
+// in psc_capi.cu.
+template <class... KA, class... A>
+inline void launch_kernel(bool pdl, void (*k)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                          const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, k, args...);
+}
 
 // X-pass modes: the right-hand side (u x omega, u . grad phi); the statistics
 // moments; the pressure inputs (u x omega and |u|^2/2 in place of the scalar term)

@@ -160,6 +160,8 @@ __device__ __forceinline__ void b_combine(const CombineArgs& c, const long long 
 }
 template <typename T, int STAGE>
 __global__ void __launch_bounds__(256) k_combine(CombineArgs c) {
+  pdl_trigger();
+  pdl_wait();
   b_combine<T, STAGE>(c, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -191,6 +193,8 @@ __global__ void __launch_bounds__(256) k_pressure(Dims d, const void* rb_, void*
 
 template <typename T>
 __global__ void __launch_bounds__(32) k_hold(Dims d, void* u_, Ctrl* ctrl, int kb, int k2max) {
+  pdl_trigger();
+  pdl_wait();
   b_hold<T>(d, u_, ctrl, kb, k2max, threadIdx.x);
 }
 template <typename T>

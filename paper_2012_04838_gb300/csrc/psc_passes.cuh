@@ -228,6 +228,7 @@ __device__ __forceinline__ void b_zinv(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT in = static_cast<const C*>(a.in);
   C* PSC_RESTRICT zb = static_cast<C*>(a.zb);
   const C* tw = strided_twiddles<T, N, W>(smraw, static_cast<const C*>(a.tw), tcx);
+  if (tcx.pdl) pdl_wait();
   const long long S = (long long)P * P * M, zs = (long long)N * P * MP;
   const C zero = mk(T(0), T(0));
   // (input field, multiply by i kz, output stream)
@@ -269,6 +270,7 @@ template <typename T, int N, bool STATS, int W, int KK = (N - 1) / 3, bool SHIFT
 __global__ void __launch_bounds__(StridedCfg<T, N, W>::THREADS, StridedCfg<T, N, W>::MINB)
 k_zinv(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  pdl_trigger();
   if (a.force.on && blockIdx.y == 0)
     return lead_force<T>(a, threadIdx.y * blockDim.x + threadIdx.x, blockDim.x * blockDim.y);
   b_zinv<T, N, STATS, W, KK, SHIFT>(a, hw_ctx(smraw, a.force.on));
@@ -287,6 +289,7 @@ __device__ __forceinline__ void b_yinv(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT zb = static_cast<const C*>(a.zb);
   C* PSC_RESTRICT yb = static_cast<C*>(a.yb);
   const C* tw = strided_twiddles<T, N, W>(smraw, static_cast<const C*>(a.tw), tcx);
+  if (tcx.pdl) pdl_wait();
   const long long zs = (long long)N * P * MP, ys = (long long)N * N * MP;
   const C zero = mk(T(0), T(0));
   // (kind, s1, s2, out): kind 0 = s1, 1 = i ky s1, 2 = i ky s1 - s2
@@ -336,6 +339,7 @@ template <typename T, int N, int YM, int W, int KK = (N - 1) / 3, bool SHIFT = f
 __global__ void __launch_bounds__(StridedCfg<T, N, W>::THREADS, StridedCfg<T, N, W>::MINB)
 k_yinv(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  pdl_trigger();
   b_yinv<T, N, YM, W, KK, SHIFT>(a, hw_ctx(smraw));
 }
 
@@ -352,6 +356,7 @@ __device__ __forceinline__ void b_yfwd(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT xb = static_cast<const C*>(a.xb);
   C* PSC_RESTRICT yf = static_cast<C*>(a.yf);
   const C* tw = strided_twiddles<T, N, W>(smraw, static_cast<const C*>(a.tw), tcx);
+  if (tcx.pdl) pdl_wait();
   const long long zs = (long long)N * P * MP, ys = (long long)N * N * MP;
   const C zero = mk(T(0), T(0));
 #pragma unroll 1
@@ -377,6 +382,7 @@ template <typename T, int N, int W, int KK = (N - 1) / 3, bool SHIFT = false>
 __global__ void __launch_bounds__(StridedCfg<T, N, W>::THREADS, StridedCfg<T, N, W>::MINB)
 k_yfwd(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  pdl_trigger();
   if (a.cfl.on && blockIdx.y == 0)
     return lead_cfl<T>(a, threadIdx.y * blockDim.x + threadIdx.x, blockDim.x * blockDim.y);
   b_yfwd<T, N, W, KK, SHIFT>(a, hw_ctx(smraw, a.cfl.on));
@@ -395,6 +401,7 @@ __device__ __forceinline__ void b_zfwd(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT yf = static_cast<const C*>(a.yf);
   C* PSC_RESTRICT rb = static_cast<C*>(a.rb);
   const C* tw = strided_twiddles<T, N, W>(smraw, static_cast<const C*>(a.tw), tcx);
+  if (tcx.pdl) pdl_wait();
   const long long S = (long long)P * P * M, zs = (long long)N * P * MP;
   const C zero = mk(T(0), T(0));
 #pragma unroll 1
@@ -420,6 +427,7 @@ template <typename T, int N, int W, int KK = (N - 1) / 3, bool SHIFT = false>
 __global__ void __launch_bounds__(StridedCfg<T, N, W>::THREADS, StridedCfg<T, N, W>::MINB)
 k_zfwd(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  pdl_trigger();
   b_zfwd<T, N, W, KK, SHIFT>(a, hw_ctx(smraw));
 }
 
@@ -614,6 +622,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
     }
     __syncthreads();
   }
+  if (tcx.pdl) pdl_wait();
   constexpr long long ys = (long long)N * N * MP;
   constexpr long long nlines = (long long)N * N;
   // every group of a warp is full: no row needs a bounds test
@@ -929,6 +938,7 @@ template <typename T, int N, int MODE, int KK = (N - 1) / 3, bool SHIFT = false>
 __global__ void __launch_bounds__(32 * XWarps<T, N>::value, xpass_ctas<T, N, MODE, (KK > (N - 1) / 3)>())
 k_xpass(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  pdl_trigger();
   b_xpass<T, N, MODE, KK, SHIFT, XWarps<T, N>::value>(a, hw_ctx(smraw));
 }
 
@@ -979,7 +989,7 @@ template <typename T, int N> struct Passes {
     using XS = XRowSmem<T, N, WR>;
     const int grid = XROW ? xrow_grid() : xwarps();
     prep(k_xrow<T, N, WR, MODE, KK, SH>, XS::SMEM);
-    k_xrow<T, N, WR, MODE, KK, SH><<<grid, XS::THREADS, XS::SMEM, a.st>>>(a);
+    launch_kernel(a.pdl != 0, k_xrow<T, N, WR, MODE, KK, SH>, grid, XS::THREADS, XS::SMEM, a.st, a);
   }
   template <int MODE, int KK, bool SH> static void xrow_k(const PassArgs& a) {
     if constexpr (XROW_OK) xrow_launch<MODE, KK, SH>(a);
@@ -1039,15 +1049,15 @@ template <typename T, int N> struct Passes {
     constexpr size_t sm = StridedSmem<T, N, W>::BYTES;
     const int gx = (M + W - 1) / W;
     const dim3 grid(gx, P + a.force.on, parts(a, gx * P, W * PlanD<N>::LPL, stats ? 8 : 7)), block(W, PlanD<N>::LPL);
-    if (stats) { prep(k_zinv<T, N, true, W>, sm); k_zinv<T, N, true, W><<<grid, block, sm, a.st>>>(a); }
-    else { prep(k_zinv<T, N, false, W>, sm); k_zinv<T, N, false, W><<<grid, block, sm, a.st>>>(a); }
+    if (stats) { prep(k_zinv<T, N, true, W>, sm); launch_kernel(a.pdl != 0, k_zinv<T, N, true, W>, grid, block, sm, a.st, a); }
+    else { prep(k_zinv<T, N, false, W>, sm); launch_kernel(a.pdl != 0, k_zinv<T, N, false, W>, grid, block, sm, a.st, a); }
   }
   template <int W, int YM> static void yinv_m(const PassArgs& a) {
     constexpr size_t sm = StridedSmem<T, N, W>::BYTES;
     const int gx = (M + W - 1) / W;
     const dim3 grid(gx, N, parts(a, gx * N, W * PlanD<N>::LPL, yinv_nt(YM))), block(W, PlanD<N>::LPL);
     prep(k_yinv<T, N, YM, W>, sm);
-    k_yinv<T, N, YM, W><<<grid, block, sm, a.st>>>(a);
+    launch_kernel(a.pdl != 0, k_yinv<T, N, YM, W>, grid, block, sm, a.st, a);
   }
   template <int W> static void yinv_w(const PassArgs& a, int ym) {
     if (ym == YMODE_STATS) yinv_m<W, YMODE_STATS>(a);
@@ -1059,14 +1069,14 @@ template <typename T, int N> struct Passes {
     const int gx = (M + W - 1) / W;
     const dim3 grid(gx, N + a.cfl.on, parts(a, gx * N, W * PlanD<N>::LPL, 4)), block(W, PlanD<N>::LPL);
     prep(k_yfwd<T, N, W>, sm);
-    k_yfwd<T, N, W><<<grid, block, sm, a.st>>>(a);
+    launch_kernel(a.pdl != 0, k_yfwd<T, N, W>, grid, block, sm, a.st, a);
   }
   template <int W> static void zfwd_w(const PassArgs& a) {
     constexpr size_t sm = StridedSmem<T, N, W>::BYTES;
     const int gx = (M + W - 1) / W;
     const dim3 grid(gx, P, parts(a, gx * P, W * PlanD<N>::LPL, 4)), block(W, PlanD<N>::LPL);
     prep(k_zfwd<T, N, W>, sm);
-    k_zfwd<T, N, W><<<grid, block, sm, a.st>>>(a);
+    launch_kernel(a.pdl != 0, k_zfwd<T, N, W>, grid, block, sm, a.st, a);
   }
   // variants 2 and 3: input tiles staged in shared memory, 4 and 8 columns (FP32)
 #ifndef PSC_STAGED
@@ -1105,7 +1115,7 @@ template <typename T, int N> struct Passes {
       const int lead = PASS == SP_ZINV ? a.force.on : PASS == SP_YFWD ? a.cfl.on : 0;
       const dim3 grid(gx, rows + lead, parts(a, gx * rows, W * PlanD<N>::LPL, StagedPlan<PASS, MODE>::NT));
       prep(k_strided_s<T, N, W, PASS, MODE>, TL::SMEM);
-      k_strided_s<T, N, W, PASS, MODE><<<grid, dim3(W, PlanD<N>::LPL), TL::SMEM, a.st>>>(a, m);
+      launch_kernel(a.pdl != 0, k_strided_s<T, N, W, PASS, MODE>, grid, dim3(W, PlanD<N>::LPL), TL::SMEM, a.st, a, m);
       return true;
     } else {
       (void)a;
@@ -1158,11 +1168,11 @@ template <typename T, int N> struct Passes {
     } else if constexpr (X2) {
       const size_t sm2 = X2Cfg<T, N>::SMEM;
       prep(k_xpass2<T, N, MODE>, sm2);
-      k_xpass2<T, N, MODE><<<xgrid(), 128, sm2, a.st>>>(a);
+      launch_kernel(a.pdl != 0, k_xpass2<T, N, MODE>, xgrid(), 128, sm2, a.st, a);
     } else {
       const size_t sm = XCfg<T, N>::smem(XW);
       prep(k_xpass<T, N, MODE>, sm);
-      k_xpass<T, N, MODE><<<xgrid(), 32 * XW, sm, a.st>>>(a);
+      launch_kernel(a.pdl != 0, k_xpass<T, N, MODE>, xgrid(), 32 * XW, sm, a.st, a);
     }
   }
   // the staged x pass of the right-hand side (rotational or convective form)
@@ -1172,7 +1182,7 @@ template <typename T, int N> struct Passes {
     const long long rows = (long long)N * N / SC::ROWS;
     const int grid = (int)(rows < sm_count() ? rows : sm_count());
     prep(k_xpass2s<T, N, KD, false, MODE>, SC::SMEM);
-    k_xpass2s<T, N, KD, false, MODE><<<grid, SC::THREADS, SC::SMEM, a.st>>>(a);
+    launch_kernel(a.pdl != 0, k_xpass2s<T, N, KD, false, MODE>, grid, SC::THREADS, SC::SMEM, a.st, a);
   }
   static void xpass_reg(const PassArgs& a, int mode) {
     if (mode == XMODE_PRESSURE) return xpass_plain<XMODE_PRESSURE>(a);
@@ -1224,7 +1234,7 @@ template <typename T, int N> struct PassesPS {
 
   template <class KER> static void go(KER k, dim3 grid, dim3 block, size_t sm, const PassArgs& a) {
     B::prep(k, sm);
-    k<<<grid, block, sm, a.st>>>(a);
+    launch_kernel(a.pdl != 0, k, grid, block, sm, a.st, a);
   }
   template <int W> static dim3 tiles(const PassArgs& a, int rows, int lead, int nt) {
     const int gx = (M + W - 1) / W;
@@ -1308,7 +1318,7 @@ template <typename T, int N> struct PassesPS {
       const int lead = PASS == SP_ZINV ? a.force.on : PASS == SP_YFWD ? a.cfl.on : 0;
       const dim3 grid(gx, rows + lead, B::parts(a, gx * rows, W * PlanD<N>::LPL, StagedPlan<PASS, MODE>::NT));
       B::prep(k_strided_s<T, N, W, PASS, MODE, KS, SH>, TL::SMEM);
-      k_strided_s<T, N, W, PASS, MODE, KS, SH><<<grid, dim3(W, PlanD<N>::LPL), TL::SMEM, a.st>>>(a, m);
+      launch_kernel(a.pdl != 0, k_strided_s<T, N, W, PASS, MODE, KS, SH>, grid, dim3(W, PlanD<N>::LPL), TL::SMEM, a.st, a, m);
       return true;
     } else {
       (void)a;
