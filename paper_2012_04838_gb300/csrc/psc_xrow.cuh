@@ -24,6 +24,8 @@ template <typename T, int N, int WR> struct XRowSmem {
   static constexpr int THREADS = 32 * WR;          // one warp per row
   static constexpr int R1 = PlanD<N>::R1, R2 = PlanD<N>::R2;
   static constexpr int RS = R2 + 1;                // exchange row stride (odd)
+  // twiddles wN^(n2 k1) as [k1][n2]: a row's lanes read consecutive entries (as
+  // wN^e, e = n2 k1, they lay k1 entries apart: up to 26 lanes on one bank)
   static constexpr size_t TW_BYTES = (size_t)N * sizeof(typename CT<T>::type);
   static constexpr size_t EX_BYTES = ((size_t)R1 * RS * sizeof(typename CT<T>::type) + 15) / 16 * 16;
   static constexpr size_t ROW_BYTES = EX_BYTES + ((size_t)NB * N * sizeof(T) + 15) / 16 * 16;
@@ -41,8 +43,8 @@ template <typename T, int N> struct XRowCfg {
   static_assert(S::SMEM <= 220 * 1024, "row buffers do not fit in shared memory");
 };
 
-// One length-N DFT of a row by one warp, direction DIR; ld(p) gives position
-// p, st(k, v) takes output k (a forward transform skips the outputs a
+// One length-N DFT of a row by one warp, direction DIR; ld(nc, n2) gives
+// position R2 nc + n2 (nc a compile-time constant), st(k, v) takes output k (a forward transform skips the outputs a
 // truncated pass drops).  Ends with __syncwarp.
 template <typename T, int N, int DIR, int KK, class LD, class ST>
 __device__ __forceinline__ void warp_row_fft(const LD& ld, const ST& st, typename CT<T>::type* ex,
@@ -55,14 +57,14 @@ __device__ __forceinline__ void warp_row_fft(const LD& ld, const ST& st, typenam
     static_for<0, R1>([&](auto nc) {
       constexpr int n1 = decltype(nc)::value;
       if constexpr (DIR > 0 && ZeroInputs<N, KK>::zero(n1)) a[n1] = mk(T(0), T(0));  // not read
-      else a[n1] = ld(R2 * n1 + n2);
+      else a[n1] = ld(nc, n2);
     });
     first_dft<T, N, DIR, KK>(a);
 #pragma unroll
     for (int k1 = 0; k1 < R1; ++k1) {
       C v = a[k1];
       if (k1 > 0) {
-        const C wv = tw[n2 * k1];  // wN^(n2 k1), n2 k1 < N
+        const C wv = tw[k1 * R2 + n2];  // wN^(n2 k1)
         v = (DIR < 0) ? cmul(v, wv) : cmulc(v, wv);
       }
       ex[k1 * RS + n2] = v;
@@ -94,7 +96,7 @@ __global__ void __launch_bounds__(XRowSmem<T, N, WR>::THREADS, 3) k_xrow(PassArg
   {
     const C* __restrict__ twg = static_cast<const C*>(a.tw);
     pdl_trigger();
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = twg[i];
+    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = twg[(i / PlanD<N>::R2) * (i % PlanD<N>::R2)];
     __syncthreads();
     pdl_wait();
   }
@@ -126,20 +128,29 @@ __global__ void __launch_bounds__(XRowSmem<T, N, WR>::THREADS, 3) k_xrow(PassArg
     // receives the two real fields at position pos.
     auto inv = [&](const auto& spec, const auto& put) {
       warp_row_fft<T, N, +1, KK>(
-          [&](int p) -> C {
+          [&](auto nc, int n2) -> C {
+            constexpr int s0 = PlanD<N>::R2 * decltype(nc)::value, band = slot_band(N, s0, PlanD<N>::R2, K);
+            const int p = s0 + n2;
             C x1, x2;
-            if (p <= K) {
+            auto low = [&]() -> C {
               spec(p, x1, x2);
               x1 = shift_in<SHIFT, KK>(x1, a.phase, p);
               x2 = shift_in<SHIFT, KK>(x2, a.phase, p);
-              if (p == 0) { x1.y = T(0); x2.y = T(0); }
+              if (s0 == 0 && p == 0) { x1.y = T(0); x2.y = T(0); }
               return mk(x1.x - x2.y, x1.y + x2.x);
-            }
-            if (p >= N - K) {
+            };
+            auto high = [&]() -> C {
               spec(N - p, x1, x2);
               x1 = shift_in<SHIFT, KK>(x1, a.phase, N - p);
               x2 = shift_in<SHIFT, KK>(x2, a.phase, N - p);
               return mk(x1.x + x2.y, x2.x - x1.y);
+            };
+            if constexpr (band == 1) {
+              if constexpr (s0 <= K) return low();
+              else return high();
+            } else if constexpr (band == 2) {
+              if (s0 <= K && p <= K) return low();
+              if (s0 + PlanD<N>::R2 > N - K && p >= N - K) return high();
             }
             return zero;
           },
@@ -151,7 +162,8 @@ __global__ void __launch_bounds__(XRowSmem<T, N, WR>::THREADS, 3) k_xrow(PassArg
     // X2 = (Z[k] - conj Z[N-k])/(2i), k <= K, go to streams s0 and s0 + 1.
     auto fwd = [&](const auto& get, int b1, int b2, int s0) {
       warp_row_fft<T, N, -1, KK>(
-          get, [&](int k, C v) { B(b1, k) = v.x; B(b2, k) = v.y; }, ex, tw, lane);
+          [&](auto nc, int n2) -> C { return get(PlanD<N>::R2 * decltype(nc)::value + n2); },
+          [&](int k, C v) { B(b1, k) = v.x; B(b2, k) = v.y; }, ex, tw, lane);
       for (int kx = lane; kx <= K; kx += 32) {
         const int kn = kx == 0 ? 0 : N - kx;
         const C A = mk(B(b1, kx), B(b2, kx)), Bn = mk(B(b1, kn), B(b2, kn));
