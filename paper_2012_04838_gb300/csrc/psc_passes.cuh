@@ -965,6 +965,9 @@ template <typename T, int N> struct Passes {
 #define PSC_X2_MIN_N 512
 #endif
   static constexpr bool X2 = (N == 512 || N == 1024) && N >= PSC_X2_MIN_N;
+  // the X pass at N = 256, 512 and 1024 (FP32) stages its rows through
+  // shared memory
+  static constexpr bool X2S = (N == 256 || X2) && sizeof(T) == 4;
   // rows whose plan gives each lane more than 64 values (N = 520: 2 lanes)
   // take the shared-memory row X pass; it also runs on request (PassArgs::xrow)
   // at the sizes with the register X pass, for testing
@@ -978,16 +981,20 @@ template <typename T, int N> struct Passes {
     return (int)(g < cap ? g : cap);
   }
   // X-pass CTAs (row X pass) or warps (register X passes) that write statistics partials
-  static int xwarps() {
+  static int xwarps_unstaged() {
     if constexpr (XROW) return xrow_grid();
     else return xgrid() * (X2 ? 4 : XW);
+  }
+  static int xwarps() {
+    if constexpr (X2S) return xstaged_grid<XMODE_STATS>() * (X2SCfg<T, N, (N - 1) / 3, XMODE_STATS>::THREADS / 32);
+    else return xwarps_unstaged();
   }
   // grid: one CTA per statistics partials slot (xwarps()) except where the
   // row X pass is the only one
   template <int MODE, int KK, bool SH> static void xrow_launch(const PassArgs& a) {
     constexpr int WR = XRC::WR;
     using XS = XRowSmem<T, N, WR>;
-    const int grid = XROW ? xrow_grid() : xwarps();
+    const int grid = XROW ? xrow_grid() : KK == PlanD<N>::K ? xwarps() : xwarps_unstaged();
     prep(k_xrow<T, N, WR, MODE, KK, SH>, XS::SMEM);
     launch_kernel(a.pdl != 0, k_xrow<T, N, WR, MODE, KK, SH>, grid, XS::THREADS, XS::SMEM, a.st, a);
   }
@@ -1159,9 +1166,6 @@ template <typename T, int N> struct Passes {
     if (v >= 2 && staged<SP_ZFWD>(a, 0, v)) return;
     v == 1 ? zfwd_w<WV1>(a) : zfwd_w<WV0>(a);
   }
-  // the right-hand side at N = 256, 512 and 1024 (FP32) stages its rows through
-  // shared memory
-  static constexpr bool X2S = (N == 256 || X2) && sizeof(T) == 4;
   template <int MODE> static void xpass_plain(const PassArgs& a) {
     if constexpr (XROW) {
       (void)a;
@@ -1175,25 +1179,21 @@ template <typename T, int N> struct Passes {
       launch_kernel(a.pdl != 0, k_xpass<T, N, MODE>, xgrid(), 32 * XW, sm, a.st, a);
     }
   }
-  // the staged x pass of the right-hand side (rotational or convective form)
+  // the staged x pass: one CTA per SM
+  template <int MODE> static int xstaged_grid() {
+    const long long rows = (long long)N * N / X2SCfg<T, N, (N - 1) / 3, MODE>::ROWS;
+    return (int)(rows < sm_count() ? rows : sm_count());
+  }
   template <int MODE> static void xpass_staged(const PassArgs& a) {
     constexpr int KD = (N - 1) / 3;
     using SC = X2SCfg<T, N, KD, MODE>;
-    const long long rows = (long long)N * N / SC::ROWS;
-    const int grid = (int)(rows < sm_count() ? rows : sm_count());
+    const int grid = xstaged_grid<MODE>();
     prep(k_xpass2s<T, N, KD, false, MODE>, SC::SMEM);
     launch_kernel(a.pdl != 0, k_xpass2s<T, N, KD, false, MODE>, grid, SC::THREADS, SC::SMEM, a.st, a);
   }
-  static void xpass_reg(const PassArgs& a, int mode) {
-    if (mode == XMODE_PRESSURE) return xpass_plain<XMODE_PRESSURE>(a);
-    if constexpr (X2S) {
-      if (mode == XMODE_RHS) return xpass_staged<XMODE_RHS>(a);
-      if (mode == XMODE_CONVECTIVE) return xpass_staged<XMODE_CONVECTIVE>(a);
-    } else {
-      if (mode == XMODE_CONVECTIVE) return xpass_plain<XMODE_CONVECTIVE>(a);
-    }
-    if (mode == XMODE_STATS) return xpass_plain<XMODE_STATS>(a);
-    if constexpr (!X2S) xpass_plain<XMODE_RHS>(a);
+  template <int MODE> static void xpass_reg(const PassArgs& a) {
+    if constexpr (X2S) xpass_staged<MODE>(a);
+    else xpass_plain<MODE>(a);
   }
   // The row X pass serves the right-hand side, the pressure inputs and the
   // statistics; the convective form needs the register X passes (it is
@@ -1207,7 +1207,12 @@ template <typename T, int N> struct Passes {
         if (mode == XMODE_RHS) return xrow_k<XMODE_RHS, K, false>(a);
       }
     }
-    if constexpr (!XROW) xpass_reg(a, mode);
+    if constexpr (!XROW) {
+      if (mode == XMODE_STATS) xpass_reg<XMODE_STATS>(a);
+      else if (mode == XMODE_PRESSURE) xpass_reg<XMODE_PRESSURE>(a);
+      else if (mode == XMODE_CONVECTIVE) xpass_reg<XMODE_CONVECTIVE>(a);
+      else xpass_reg<XMODE_RHS>(a);
+    }
   }
   static const PassTable* table() {
     static const PassTable tb = {&zinv, &yinv, &xpass, &yfwd, &zfwd,
@@ -1377,7 +1382,7 @@ template <typename T, int N> struct PassesPS {
   }
   static const PassTable* table() {
     static const PassTable tb = {&zinv, &yinv, &xpass, &yfwd, &zfwd,
-                                 B::xwarps(), NVS,
+                                 B::xwarps_unstaged(), NVS,
                                  {WV0, WV1, 4, 8, 16}, {0, 0, 1, 1, 1},
                                  {MASK_INV, MASK_INV, MASK_FWD, MASK_FWD}, ROWS ? 1 : 0};
     return &tb;

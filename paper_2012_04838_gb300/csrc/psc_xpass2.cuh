@@ -478,6 +478,91 @@ __device__ __forceinline__ bool x2_conv_row(const YF& Y, const HA& after_a, cons
   return true;
 }
 
+// The statistics of one row (Eqs. 11-13): each pair's moments over the thread's 16
+// points are added up plainly and join the thread's compensated sums.  The hooks
+// as in x2_rhs_row: after_a() once all streams but DYPHI, DZPHI and DZUZ are no
+// longer read, wait_b() before those are, after_b() once they are not.
+template <typename T, int N, int KK, class YF, class HA, class WB, class HB>
+__device__ __forceinline__ bool x2_stats_row(const YF& Y, const HA& after_a, const WB& wait_b, const HB& after_b,
+                                             typename CT<T>::type* ex, const X2Roles<typename CT<T>::type>& q, T scale,
+                                             MomentSum<T> (&acc)[NQ], T& um) {
+  using C = typename CT<T>::type;
+  const C zero = mk(T(0), T(0));
+  C z[16];
+  T s13[16];
+  auto mom3 = [&](int slot, auto&& f) {
+    T m2 = T(0), m3 = T(0), m4 = T(0);
+#pragma unroll
+    for (int b = 0; b < 16; ++b) { const T v = f(b), v2 = v * v; m2 += v2; m3 += v2 * v; m4 += v2 * v2; }
+    acc[slot].add(m2);
+    acc[slot + 1].add(m3);
+    acc[slot + 2].add(m4);
+  };
+  auto re = [&](int b) { return z[b].x; };
+  auto im = [&](int b) { return z[b].y; };
+  // (u1, u3)
+  x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UZ, kx); }, z, ex, q, scale);
+  {
+    T s = T(0);
+#pragma unroll
+    for (int b = 0; b < 16; ++b) { s += z[b].x * z[b].x + z[b].y * z[b].y; s13[b] = fabs(z[b].x) + fabs(z[b].y); }
+    acc[0].add(s);
+  }
+  // (u2, phi)
+  x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UY, kx); x2 = Y(Y_PHI, kx); }, z, ex, q, scale);
+  {
+    T s0 = T(0), s1 = T(0), s2 = T(0);
+#pragma unroll
+    for (int b = 0; b < 16; ++b) {
+      s0 += z[b].x * z[b].x; s1 += z[b].y * z[b].x; s2 += z[b].y * z[b].y;
+      um = max_keep_nan(um, s13[b] + fabs(z[b].x));
+    }
+    acc[0].add(s0);
+    acc[20].add(s1);
+    acc[21].add(s2);
+  }
+  // (omega1, omega2)
+  x2inv<T, N, true, KK>(
+      [&](int kx, C& x1, C& x2) { x1 = Y(Y_WX, kx); x2 = csub(Y(Y_DZUX, kx), mul_ik(Y(Y_UZ, kx), T(kx))); }, z, ex, q,
+      scale);
+  {
+    T s = T(0);
+#pragma unroll
+    for (int b = 0; b < 16; ++b) s += z[b].x * z[b].x + z[b].y * z[b].y;
+    acc[1].add(s);
+  }
+  // (omega3, dphi/dx1)
+  x2inv<T, N, true, KK>(
+      [&](int kx, C& x1, C& x2) {
+        x1 = csub(mul_ik(Y(Y_UY, kx), T(kx)), Y(Y_DYUX, kx));
+        x2 = mul_ik(Y(Y_PHI, kx), T(kx));
+      },
+      z, ex, q, scale);
+  {
+    T s = T(0);
+#pragma unroll
+    for (int b = 0; b < 16; ++b) s += z[b].x * z[b].x;
+    acc[1].add(s);
+    mom3(11, im);
+  }
+  // (du1/dx1, du2/dx2)
+  x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_UX, kx), T(kx)); x2 = Y(Y_DYUY, kx); }, z, ex, q,
+                        scale);
+  after_a();
+  mom3(2, re);
+  mom3(5, im);
+  if (!wait_b()) return false;
+  // (dphi/dx2, dphi/dx3)
+  x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DYPHI, kx); x2 = Y(Y_DZPHI, kx); }, z, ex, q, scale);
+  mom3(14, re);
+  mom3(17, im);
+  // (du3/dx3, 0)
+  x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZUZ, kx); x2 = zero; }, z, ex, q, scale);
+  after_b();
+  mom3(8, re);
+  return true;
+}
+
 template <typename T>
 __device__ __forceinline__ double warp_sum_d(T v) {
   double d = (double)v;
@@ -528,7 +613,6 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : PSC_X2_MINB) k_xpass
       if (!PSC_OK_INDEX(s * ys + line * MP + kx, (long long)Y_NSTREAM * ys, a.ctrl)) return zero;
       return row[s * ys + kx];
     };
-    C z[16];
     if constexpr (MODE == XMODE_RHS || MODE == XMODE_PRESSURE) {
       x2_rhs_row<T, N, MODE == XMODE_PRESSURE, KK, SHIFT>(Y, [] {}, [] { return true; }, [] {}, xb, line, ys, ex, q,
                                                           scale, a.want_umax != 0, um, a.ctrl, a.phase);
@@ -536,84 +620,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : PSC_X2_MINB) k_xpass
       x2_conv_row<T, N, KK, SHIFT>(Y, [] {}, [] { return true; }, [] {}, xb, line, ys, ex, q, scale,
                                    a.want_umax != 0, um, a.ctrl, a.phase);
     } else {
-      // statistics (Eqs. 11-13): per pair, partial sums of the thread's 16
-      // points, added in FP64 to the thread's accumulators (reduced over the
-      // warp once, at the end)
-      T s13[16];
-      auto put = [&](int slot, T v) { acc[slot].add(v); };
-      auto mom3 = [&](int slot, const T (&f)[16]) {
-        T m2 = T(0), m3 = T(0), m4 = T(0);
-#pragma unroll
-        for (int b = 0; b < 16; ++b) { const T v2 = f[b] * f[b]; m2 += v2; m3 += v2 * f[b]; m4 += v2 * v2; }
-        put(slot, m2); put(slot + 1, m3); put(slot + 2, m4);
-      };
-      T f1[16], f2[16];
-      auto split = [&]() {
-#pragma unroll
-        for (int b = 0; b < 16; ++b) { f1[b] = z[b].x; f2[b] = z[b].y; }
-      };
-      // (u1, u3)
-      x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UZ, kx); }, z, ex, q, scale);
-      split();
-      {
-        T s = T(0);
-#pragma unroll
-        for (int b = 0; b < 16; ++b) { s += f1[b] * f1[b] + f2[b] * f2[b]; s13[b] = fabs(f1[b]) + fabs(f2[b]); }
-        put(0, s);
-      }
-      // (u2, phi)
-      x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UY, kx); x2 = Y(Y_PHI, kx); }, z, ex, q, scale);
-      split();
-      {
-        T s0 = T(0), s1 = T(0), s2 = T(0);
-#pragma unroll
-        for (int b = 0; b < 16; ++b) {
-          s0 += f1[b] * f1[b]; s1 += f2[b] * f1[b]; s2 += f2[b] * f2[b];
-          um = max_keep_nan(um, s13[b] + fabs(f1[b]));
-        }
-        put(0, s0); put(20, s1); put(21, s2);
-      }
-      // (omega1, omega2)
-      x2inv<T, N, true, KK>(
-          [&](int kx, C& x1, C& x2) { x1 = Y(Y_WX, kx); x2 = csub(Y(Y_DZUX, kx), mul_ik(Y(Y_UZ, kx), T(kx))); },
-          z, ex, q, scale);
-      split();
-      {
-        T s = T(0);
-#pragma unroll
-        for (int b = 0; b < 16; ++b) s += f1[b] * f1[b] + f2[b] * f2[b];
-        put(1, s);
-      }
-      // (omega3, dphi/dx1)
-      x2inv<T, N, true, KK>(
-          [&](int kx, C& x1, C& x2) {
-            x1 = csub(mul_ik(Y(Y_UY, kx), T(kx)), Y(Y_DYUX, kx));
-            x2 = mul_ik(Y(Y_PHI, kx), T(kx));
-          },
-          z, ex, q, scale);
-      split();
-      {
-        T s = T(0);
-#pragma unroll
-        for (int b = 0; b < 16; ++b) s += f1[b] * f1[b];
-        put(1, s);
-        mom3(11, f2);
-      }
-      // (dphi/dx2, dphi/dx3)
-      x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DYPHI, kx); x2 = Y(Y_DZPHI, kx); }, z, ex, q, scale);
-      split();
-      mom3(14, f1);
-      mom3(17, f2);
-      // (du1/dx1, du2/dx2)
-      x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_UX, kx), T(kx)); x2 = Y(Y_DYUY, kx); }, z, ex,
-                  q, scale);
-      split();
-      mom3(2, f1);
-      mom3(5, f2);
-      // (du3/dx3, 0)
-      x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZUZ, kx); x2 = zero; }, z, ex, q, scale);
-      split();
-      mom3(8, f1);
+      x2_stats_row<T, N, KK>(Y, [] {}, [] { return true; }, [] {}, ex, q, scale, acc, um);
     }
   }
 
@@ -639,8 +646,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : PSC_X2_MINB) k_xpass
 }
 
 // ---------------------------------------------------------------------------
-// Staged x pass (right-hand side, rotational or convective form; FP32, N = 256,
-// 512 and 1024).  One CTA per SM holds X2SCfg::UNITS units in flight, a unit
+// Staged x pass (the right-hand side in either form, the pressure inputs and the
+// statistics; FP32, N = 256, 512 and 1024).  One CTA per SM holds X2SCfg::UNITS units in flight, a unit
 // being a row, or the two adjacent rows of a warp at N = 256; the input streams
 // of each unit are copied into shared memory by bulk asynchronous copies (TMA
 // engine) one unit ahead, in two groups completed on two mbarriers:
@@ -669,6 +676,18 @@ template <> struct X2SGroups<XMODE_CONVECTIVE> {
                                 (1u << Y_DYUY) | (1u << Y_DZUY);
   static constexpr unsigned B = (1u << Y_WX) | (1u << Y_PHI) | (1u << Y_DYPHI) | (1u << Y_DZPHI) | (1u << Y_DZUZ);
   static constexpr int SLOTS = Y_DZUY + 1;
+};
+template <> struct X2SGroups<XMODE_PRESSURE> {
+  // the right-hand side's first group; the pressure inputs need no more
+  static constexpr unsigned A = X2SGroups<XMODE_RHS>::A;
+  static constexpr unsigned B = 0;
+  static constexpr int SLOTS = Y_DYUX + 1;
+};
+template <> struct X2SGroups<XMODE_STATS> {
+  // all but the last two transforms' streams, and those
+  static constexpr unsigned B = (1u << Y_DYPHI) | (1u << Y_DZPHI) | (1u << Y_DZUZ);
+  static constexpr unsigned A = ((1u << (Y_DZUZ + 1)) - 1u) & ~B;
+  static constexpr int SLOTS = Y_DZUZ + 1;
 };
 
 template <typename T, int N, int KK = (N - 1) / 3, int MODE = XMODE_RHS> struct X2SCfg {
@@ -715,7 +734,6 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
   using SC = X2SCfg<T, N, KK, MODE>;
   using G = typename SC::G;
   static_assert(SC::OK, "staged x pass: rows must be 16-byte multiples and fit shared memory");
-  static_assert(MODE == XMODE_RHS || MODE == XMODE_CONVECTIVE, "staged x pass: right-hand side only");
   constexpr int TH = XC::TH, G_ = XC::G, MP = SC::MP, RPU = SC::RPU, UTH = SC::UTH, UNITS = SC::UNITS;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int uid = threadIdx.x / UTH, sub = threadIdx.x % UTH / TH;  // unit, and row within it
@@ -765,6 +783,7 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
     }
   };
   T um = T(0);
+  MomentSum<T> acc[MODE == XMODE_STATS ? NQ : 1];
   unsigned pa = 0, pb = 0;        // parity of the next phase to wait for
   bool ia = false, ib = false;    // a group issued and not yet waited for
   bool ok = true;
@@ -772,10 +791,11 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
   if (line < nlines) {
     if (leader) {
       issue(line, G::A, barA);
-      issue(line, G::B, barB);
+      if (G::B) issue(line, G::B, barB);
     }
     __syncwarp();
-    ia = ib = true;
+    ia = true;
+    ib = G::B != 0;
   }
 #pragma unroll 1
   for (; line < nlines; line += stride) {
@@ -812,8 +832,10 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
         ib = true;
       }
     };
-    if constexpr (MODE == XMODE_RHS)
-      ok = x2_rhs_row<T, N, false, KK, SHIFT>(Y, after_a, wait_b, after_b, xb, line + sub, ys, ex, q, scale,
+    if constexpr (MODE == XMODE_STATS)
+      ok = x2_stats_row<T, N, KK>(Y, after_a, wait_b, after_b, ex, q, scale, acc, um);
+    else if constexpr (MODE != XMODE_CONVECTIVE)
+      ok = x2_rhs_row<T, N, MODE == XMODE_PRESSURE, KK, SHIFT>(Y, after_a, wait_b, after_b, xb, line + sub, ys, ex, q, scale,
                                               a.want_umax != 0, um, a.ctrl, a.phase);
     else
       ok = x2_conv_row<T, N, KK, SHIFT>(Y, after_a, wait_b, after_b, xb, line + sub, ys, ex, q, scale,
@@ -829,13 +851,21 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
       if (ib) mbar_wait(barB, pb, nullptr, lim);
     }
   }
-  if (a.want_umax) {
-    double umax = (double)um * (double)scale;
+  if (MODE == XMODE_STATS || a.want_umax) {
+    double umax = MODE == XMODE_STATS ? (double)um : (double)um * (double)scale;
     for (int o = 16; o > 0; o >>= 1) {
       const double other = __shfl_xor_sync(0xffffffffu, umax, o);
       umax = other > umax || other != other ? other : umax;
     }
     if ((threadIdx.x & 31) == 0) atomicMax(&a.ctrl->umax_bits, (unsigned long long)__double_as_longlong(umax));
+  }
+  if constexpr (MODE == XMODE_STATS) {
+    const long long gw = (long long)blockIdx.x * (SC::THREADS / 32) + threadIdx.x / 32;
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      const double v = warp_sum_d<double>(acc[i].value());
+      if ((threadIdx.x & 31) == 0) a.partials[gw * NQ + i] = v;
+    }
   }
 }
 
