@@ -564,19 +564,22 @@ CombineArgs combine_args(psc_sim* s, const void* vin) {
   return c;
 }
 
+template <typename T, bool PDL>
+void combine_stage(int stage, int blocks, cudaStream_t st, const CombineArgs& c) {
+  switch (stage) {
+    case 0: launch_kernel(PDL, k_combine<T, 0, PDL>, blocks, 256, 0, st, c); break;
+    case 1: launch_kernel(PDL, k_combine<T, 1, PDL>, blocks, 256, 0, st, c); break;
+    case 2: launch_kernel(PDL, k_combine<T, 2, PDL>, blocks, 256, 0, st, c); break;
+    case 3: launch_kernel(PDL, k_combine<T, 3, PDL>, blocks, 256, 0, st, c); break;
+    default: launch_kernel(PDL, k_combine<T, 4, PDL>, blocks, 256, 0, st, c); break;
+  }
+}
 template <typename T>
 void launch_combine(psc_sim* s, int stage, const CombineArgs& c) {
-  const long long S = s->d.S;
-  const int blocks = (int)((S + 255) / 256);
+  const int blocks = (int)((s->d.S + 255) / 256);
   launch(s, PSC_K_COMBINE, 1, [&] {
-    const bool pdl = s->pdl != 0;
-    switch (stage) {
-      case 0: launch_kernel(pdl, k_combine<T, 0>, blocks, 256, 0, s->st, c); break;
-      case 1: launch_kernel(pdl, k_combine<T, 1>, blocks, 256, 0, s->st, c); break;
-      case 2: launch_kernel(pdl, k_combine<T, 2>, blocks, 256, 0, s->st, c); break;
-      case 3: launch_kernel(pdl, k_combine<T, 3>, blocks, 256, 0, s->st, c); break;
-      default: launch_kernel(pdl, k_combine<T, 4>, blocks, 256, 0, s->st, c); break;
-    }
+    if (s->pdl) combine_stage<T, true>(stage, blocks, s->st, c);
+    else combine_stage<T, false>(stage, blocks, s->st, c);
   });
 }
 
@@ -621,7 +624,7 @@ psc_status do_step(psc_sim* s, int nsteps) {
     if (s->p.forcing == PSC_FORCE_HOLD_ENERGY) {
       launch(s, PSC_K_FORCING, 1, [&] {
         const ForceArgs f = force_args(s, false, false);
-        launch_kernel(s->pdl != 0, k_hold<T>, 1, 32, 0, s->st, s->d, (void*)U, s->ctrl, f.kb, f.k2max);
+        launch_kernel(s->pdl != 0, k_hold<T>, 1, 32, 0, s->st, s->d, (void*)U, s->ctrl, f.kb, f.k2max, s->pdl);
       });
     }
     PSC_LAUNCHED("psc_step");

@@ -97,10 +97,14 @@ template <int N> struct PlanD : Plan<N> {
 // the stream drains (launch_kernel), so its CTAs start, and fill their twiddle
 // tables, beside the last CTAs of that pass.  pdl_wait() returns once every
 // earlier kernel of the stream has completed and its writes are visible, and
-// comes before the first access to anything those kernels write; without the
-// launch attribute it returns at once.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// comes before the first access to anything those kernels write.
+// (`on`: the launch has the attribute.)
+__device__ __forceinline__ void pdl_trigger(int on) {
+  if (on) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait(int on) {
+  if (on) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 
 // Thread and block coordinates of a kernel body: the hardware's in an ordinary
 // launch, or virtual ones when the persistent ensemble kernel runs the body as
@@ -110,12 +114,11 @@ struct Tctx {
   int tx, ty, bx, by, bdx, bdy, gdx;
   unsigned char* smem;  // the body's dynamic shared memory
   int part = 0, parts = 1;
-  bool pdl = false;  // an ordinary launch: wait for the kernels before it
 };
 // lead: rows of CTAs ahead of the pass's own (PassArgs::force, PassArgs::cfl)
 __device__ __forceinline__ Tctx hw_ctx(unsigned char* smem, int lead = 0) {
   return Tctx{(int)threadIdx.x, (int)threadIdx.y, (int)blockIdx.x, (int)blockIdx.y - lead,
-              (int)blockDim.x,  (int)blockDim.y,  (int)gridDim.x,  smem, (int)blockIdx.z, (int)gridDim.z, true};
+              (int)blockDim.x,  (int)blockDim.y,  (int)gridDim.x,  smem, (int)blockIdx.z, (int)gridDim.z};
 }
 // Grids whose strided passes may be cut into shares (Passes::parts): above 256
 // the tiles alone always fill the chip, and the loop bounds stay constants.

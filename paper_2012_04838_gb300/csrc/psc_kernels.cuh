@@ -158,10 +158,15 @@ __device__ __forceinline__ void b_combine(const CombineArgs& c, const long long 
     }
   }
 }
-template <typename T, int STAGE>
+// PDL: launched as a programmatic dependent; a template parameter, because the
+// wait's memory clobber in an otherwise plain kernel costs it 5% at 1024^3 (3.36 ->
+// 3.54 ms a launch)
+template <typename T, int STAGE, bool PDL>
 __global__ void __launch_bounds__(256) k_combine(CombineArgs c) {
-  pdl_trigger();
-  pdl_wait();
+  if constexpr (PDL) {
+    pdl_trigger(1);
+    pdl_wait(1);
+  }
   b_combine<T, STAGE>(c, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -192,9 +197,9 @@ __global__ void __launch_bounds__(256) k_pressure(Dims d, const void* rb_, void*
 }
 
 template <typename T>
-__global__ void __launch_bounds__(32) k_hold(Dims d, void* u_, Ctrl* ctrl, int kb, int k2max) {
-  pdl_trigger();
-  pdl_wait();
+__global__ void __launch_bounds__(32) k_hold(Dims d, void* u_, Ctrl* ctrl, int kb, int k2max, int pdl) {
+  pdl_trigger(pdl);
+  pdl_wait(pdl);
   b_hold<T>(d, u_, ctrl, kb, k2max, threadIdx.x);
 }
 template <typename T>

@@ -228,7 +228,7 @@ __device__ __forceinline__ void b_zinv(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT in = static_cast<const C*>(a.in);
   C* PSC_RESTRICT zb = static_cast<C*>(a.zb);
   const C* tw = strided_twiddles<T, N, W>(smraw, static_cast<const C*>(a.tw), tcx);
-  if (tcx.pdl) pdl_wait();
+  pdl_wait(a.pdl);
   const long long S = (long long)P * P * M, zs = (long long)N * P * MP;
   const C zero = mk(T(0), T(0));
   // (input field, multiply by i kz, output stream)
@@ -270,7 +270,7 @@ template <typename T, int N, bool STATS, int W, int KK = (N - 1) / 3, bool SHIFT
 __global__ void __launch_bounds__(StridedCfg<T, N, W>::THREADS, StridedCfg<T, N, W>::MINB)
 k_zinv(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  pdl_trigger();
+  pdl_trigger(a.pdl);
   if (a.force.on && blockIdx.y == 0)
     return lead_force<T>(a, threadIdx.y * blockDim.x + threadIdx.x, blockDim.x * blockDim.y);
   b_zinv<T, N, STATS, W, KK, SHIFT>(a, hw_ctx(smraw, a.force.on));
@@ -289,7 +289,7 @@ __device__ __forceinline__ void b_yinv(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT zb = static_cast<const C*>(a.zb);
   C* PSC_RESTRICT yb = static_cast<C*>(a.yb);
   const C* tw = strided_twiddles<T, N, W>(smraw, static_cast<const C*>(a.tw), tcx);
-  if (tcx.pdl) pdl_wait();
+  pdl_wait(a.pdl);
   const long long zs = (long long)N * P * MP, ys = (long long)N * N * MP;
   const C zero = mk(T(0), T(0));
   // (kind, s1, s2, out): kind 0 = s1, 1 = i ky s1, 2 = i ky s1 - s2
@@ -339,7 +339,7 @@ template <typename T, int N, int YM, int W, int KK = (N - 1) / 3, bool SHIFT = f
 __global__ void __launch_bounds__(StridedCfg<T, N, W>::THREADS, StridedCfg<T, N, W>::MINB)
 k_yinv(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  pdl_trigger();
+  pdl_trigger(a.pdl);
   b_yinv<T, N, YM, W, KK, SHIFT>(a, hw_ctx(smraw));
 }
 
@@ -356,7 +356,7 @@ __device__ __forceinline__ void b_yfwd(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT xb = static_cast<const C*>(a.xb);
   C* PSC_RESTRICT yf = static_cast<C*>(a.yf);
   const C* tw = strided_twiddles<T, N, W>(smraw, static_cast<const C*>(a.tw), tcx);
-  if (tcx.pdl) pdl_wait();
+  pdl_wait(a.pdl);
   const long long zs = (long long)N * P * MP, ys = (long long)N * N * MP;
   const C zero = mk(T(0), T(0));
 #pragma unroll 1
@@ -382,7 +382,7 @@ template <typename T, int N, int W, int KK = (N - 1) / 3, bool SHIFT = false>
 __global__ void __launch_bounds__(StridedCfg<T, N, W>::THREADS, StridedCfg<T, N, W>::MINB)
 k_yfwd(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  pdl_trigger();
+  pdl_trigger(a.pdl);
   if (a.cfl.on && blockIdx.y == 0)
     return lead_cfl<T>(a, threadIdx.y * blockDim.x + threadIdx.x, blockDim.x * blockDim.y);
   b_yfwd<T, N, W, KK, SHIFT>(a, hw_ctx(smraw, a.cfl.on));
@@ -401,7 +401,7 @@ __device__ __forceinline__ void b_zfwd(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT yf = static_cast<const C*>(a.yf);
   C* PSC_RESTRICT rb = static_cast<C*>(a.rb);
   const C* tw = strided_twiddles<T, N, W>(smraw, static_cast<const C*>(a.tw), tcx);
-  if (tcx.pdl) pdl_wait();
+  pdl_wait(a.pdl);
   const long long S = (long long)P * P * M, zs = (long long)N * P * MP;
   const C zero = mk(T(0), T(0));
 #pragma unroll 1
@@ -427,7 +427,7 @@ template <typename T, int N, int W, int KK = (N - 1) / 3, bool SHIFT = false>
 __global__ void __launch_bounds__(StridedCfg<T, N, W>::THREADS, StridedCfg<T, N, W>::MINB)
 k_zfwd(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  pdl_trigger();
+  pdl_trigger(a.pdl);
   b_zfwd<T, N, W, KK, SHIFT>(a, hw_ctx(smraw));
 }
 
@@ -622,7 +622,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
     }
     __syncthreads();
   }
-  if (tcx.pdl) pdl_wait();
+  pdl_wait(a.pdl);
   constexpr long long ys = (long long)N * N * MP;
   constexpr long long nlines = (long long)N * N;
   // every group of a warp is full: no row needs a bounds test
@@ -938,7 +938,7 @@ template <typename T, int N, int MODE, int KK = (N - 1) / 3, bool SHIFT = false>
 __global__ void __launch_bounds__(32 * XWarps<T, N>::value, xpass_ctas<T, N, MODE, (KK > (N - 1) / 3)>())
 k_xpass(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  pdl_trigger();
+  pdl_trigger(a.pdl);
   b_xpass<T, N, MODE, KK, SHIFT, XWarps<T, N>::value>(a, hw_ctx(smraw));
 }
 

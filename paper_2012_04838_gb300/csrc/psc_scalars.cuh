@@ -116,13 +116,13 @@ __device__ __forceinline__ void b_cfl(Ctrl* c, double cfl, double dx, int record
 template <typename T>
 __device__ __forceinline__ void lead_force(const PassArgs& a, int me, int nthr) {
   const int lanes = nthr < 32 ? nthr : 32;
-  pdl_wait();
+  pdl_wait(a.pdl);
   if (blockIdx.x == 0 && blockIdx.z == 0 && me < lanes) b_famp<T>(a.d, a.in, a.ctrl, a.force, me, lanes);
 }
 template <typename T>
 __device__ __forceinline__ void lead_cfl(const PassArgs& a, int me, int nthr) {
   if (blockIdx.x != 0 || blockIdx.z != 0) return;
-  pdl_wait();
+  pdl_wait(a.pdl);
   if (me == 0) b_cfl(a.ctrl, a.cfl.cfl, a.cfl.dx, a.cfl.record_every);
   __syncthreads();
   for (int k = me; k <= a.d.K; k += nthr)

@@ -212,7 +212,7 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
   using SPL = StagedPlan<PASS, MODE>;
   constexpr int K = KK, M = KK + 1, MP = row_pitch(M), P = 2 * KK + 1, R1 = PL::R1, R2 = PL::R2, TPL = PL::TPL, NJ1 = PlanD<N>::SJ1;
   extern __shared__ __align__(16) unsigned char smraw[];
-  pdl_trigger();
+  pdl_trigger(a.pdl);
   C* sm = reinterpret_cast<C*>(smraw);
   C* stg = reinterpret_cast<C*>(smraw + TL::STG_OFF);
   unsigned long long* bar = reinterpret_cast<unsigned long long*>(smraw + TL::BAR_OFF);
@@ -262,7 +262,7 @@ k_strided_s(PassArgs a, const __grid_constant__ CUtensorMap tm) {
     tw = static_cast<const C*>(a.tw);
   }
   __syncthreads();  // barrier initialised and twiddles in place before use
-  pdl_wait();
+  pdl_wait(a.pdl);
   const long long S = (long long)P * P * M, zs = (long long)N * P * MP, ys = (long long)N * N * MP;
   const C* __restrict__ cin = static_cast<const C*>(a.in);
   auto issue = [&](int tr) {

@@ -592,9 +592,9 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : PSC_X2_MINB) k_xpass
   const C* __restrict__ yb = static_cast<const C*>(a.yb);
   C* __restrict__ xb = static_cast<C*>(a.xb);
   const C* __restrict__ tw = static_cast<const C*>(a.tw);
-  pdl_trigger();
+  pdl_trigger(a.pdl);
   x2_twiddles<T, N>(reinterpret_cast<C*>(smraw + XC::LINE_BYTES * ROWS + XC::ACC_BYTES), tw, q);
-  pdl_wait();
+  pdl_wait(a.pdl);
   // rows and the stream stride come from the arguments (N*N rows for a pass over the box)
   const long long ys = a.d.ys;
   const long long nlines = ys / MP;
@@ -756,9 +756,9 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
     mbar_init(barB, 1);
     mbar_init_fence();
   }
-  pdl_trigger();
+  pdl_trigger(a.pdl);
   x2_twiddles<T, N>(reinterpret_cast<C*>(smraw + SC::TW_OFF), static_cast<const C*>(a.tw), q);
-  pdl_wait();
+  pdl_wait(a.pdl);
   const long long ys = a.d.ys;  // N*N*MP for a pass over the box
   const long long nlines = ys / MP;
   const long long stride = (long long)gridDim.x * SC::ROWS;

@@ -95,10 +95,10 @@ __global__ void __launch_bounds__(XRowSmem<T, N, WR>::THREADS, 3) k_xrow(PassArg
   C* tw = reinterpret_cast<C*>(smraw);
   {
     const C* __restrict__ twg = static_cast<const C*>(a.tw);
-    pdl_trigger();
+    pdl_trigger(a.pdl);
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = twg[(i / PlanD<N>::R2) * (i % PlanD<N>::R2)];
     __syncthreads();
-    pdl_wait();
+    pdl_wait(a.pdl);
   }
   unsigned char* myrow = smraw + XS::TW_BYTES + (size_t)wid * XS::ROW_BYTES;
   C* ex = reinterpret_cast<C*>(myrow);
