@@ -192,9 +192,10 @@ psc_status psc_time(psc_sim* s, double* t, int64_t* step, double* dt);
 /* Ensembles (boxes of any mix of N and precision stepped together).
  *
  * psc_batch_create() captures one RK4 step of every member into a single CUDA
- * graph, each member on its own stream as a parallel branch forked from and
- * joined back into `stream`; psc_batch_step() replays that graph, so an
- * ensemble step costs one graph launch and small boxes run concurrently.
+ * graph, each member's work on its own stream, forked from and joined back into
+ * `stream`; psc_batch_step() replays that graph, so an ensemble step costs one
+ * graph launch and small boxes run concurrently (the largest first, as many at a
+ * time as fit a budget of workspace bytes).
  * Each member advances exactly as psc_step() would advance it (the step counter
  * and the CFL decision live on the device).  Members need non-NULL streams;
  * members that share a stream become consecutive steps of one branch (correct,
@@ -250,14 +251,15 @@ psc_status psc_batch_info(const psc_batch* b, int32_t* mode, int32_t* grid, int6
 
 /* Kernel classes for profiling. */
 typedef enum {
-  PSC_K_FORCING = 0,  /* band energy and forcing amplitude                   */
+  PSC_K_FORCING = 0,  /* deterministic forcing's rescaling (the amplitude is
+                         taken within the z-inverse launch)                  */
   PSC_K_ZINV = 1,     /* inverse transform along z (+ d/dz streams)          */
   PSC_K_YINV = 2,     /* inverse transform along y (+ omega_x, d/dy streams) */
   PSC_K_XPASS = 3,    /* fused x transforms and nonlinear products           */
   PSC_K_YFWD = 4,     /* forward transform along y, truncation               */
   PSC_K_ZFWD = 5,     /* forward transform along z, truncation               */
   PSC_K_COMBINE = 6,  /* projection, forcing, scalar source, RK stage update */
-  PSC_K_OTHER = 7,    /* CFL, IF tables, statistics passes and reductions, IC */
+  PSC_K_OTHER = 7,    /* statistics passes and reductions, IC                */
   PSC_K_NKIND = 8
 } psc_kernel_kind;
 

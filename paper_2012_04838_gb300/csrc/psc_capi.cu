@@ -784,7 +784,7 @@ psc_status do_stats(psc_sim* s, double* Ek, double* Ephi, int cap, int* nshell, 
 }
 
 // Autotuner of the strided passes.  Every compiled variant of each pass (tile
-// widths, and for FP32 grids with an even M the TMA-staged kernels) is timed
+// widths, and for FP32 grids of 64 and more the staged kernels) is timed
 // on this simulation's own workspace (one warm-up and three timed launches
 // each, CUDA events on its stream) and the fastest is kept.
 // Choices are cached per (grid size, precision) for the life of the process,

@@ -11,7 +11,7 @@ member's kernels into one CUDA graph per RK4 step, rebuilt when the set
 changes; "persistent" steps it with one persistent launch per RK stage over a
 device work table that is rewritten when runs join or leave, so nothing is
 recaptured (FP32-mixed runs at the persistent sizes; on GB300 it has run at
-about half the graph path's rate, its pass bodies being latency-bound at the
+about 0.6 of the graph path's rate, its pass bodies being latency-bound at the
 occupancy one kernel for every pass allows).  While a chunk of steps runs on
 the GPU the host admits and initialises newly arrived runs.
 
