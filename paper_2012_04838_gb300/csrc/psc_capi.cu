@@ -168,6 +168,7 @@ struct psc_sim {
   int64_t step;
   int nshell;
   int wv[SP_N];  // tile-width variant of each strided pass (autotuned at creation)
+  bool tuned = false;  // wv was measured (not forced by the environment)
   int xrow = 0;  // PSC_XPASS_ROWS=1 at creation: the row X pass where the register one exists
   int stall_test = 0;  // PSC_XPASS_STALL_TEST=1 at creation: failure-path test of the TMA waits
   int pdl = 0;    // programmatic dependent launches (psc_create; off inside a batch's graph, whose branches fill the chip)
@@ -826,6 +827,7 @@ psc_status autotune(psc_sim* s) {
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
       for (int p = 0; p < SP_N; ++p) s->wv[p] = it->second[p];
+      s->tuned = true;
       return PSC_OK;
     }
   }
@@ -866,6 +868,7 @@ psc_status autotune(psc_sim* s) {
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "psc_create: tile autotuning");
   for (int p = 0; p < SP_N; ++p) s->wv[p] = best[p];
+  s->tuned = true;
   std::lock_guard<std::mutex> lock(g_tune_mu);
   g_tune_cache[key] = best;
   return PSC_OK;
@@ -1140,6 +1143,16 @@ psc_status psc_batch_create(psc_sim* const* sims, int32_t n, void* stream, psc_b
   // once 4.92; 20 / 60 / 110 / 180 / 240 / 400 / 1000 MB under way 8.92 / 5.84 /
   // 4.82 / 4.61 / 4.37 / 4.35 / 4.59.
   constexpr size_t kBatchBytes = (size_t)320 << 20;
+  // The tile variants were measured with a box alone on the chip.  Where the
+  // members keep the chip full instead (their workspaces exceed what is let under
+  // way), the staged 8-column variant is faster in every strided pass than the
+  // measured mixture, whose wider and unstaged tiles pay by filling idle SMs:
+  // us a step, measured mixture -> staged, 48 x 64^3 + 12 x 96^3 + 3 x 128^3
+  // 4357 -> 4249, 24 x 64^3 943 -> 926, 8 x 96^3 1077 -> 1050, 3 x 128^3 1045 ->
+  // 1030; 4 x 64^3, which leave room, 172 -> 175.  All variants give the same bits.
+  size_t total = 0;
+  for (int i = 0; i < n; ++i) total += sims[i]->L.total;
+  const bool full = total > kBatchBytes;
   std::vector<int> order(n);
   for (int i = 0; i < n; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return sims[x]->L.total > sims[y]->L.total; });
@@ -1172,7 +1185,14 @@ psc_status psc_batch_create(psc_sim* const* sims, int32_t n, void* stream, psc_b
     used += m->L.total;
     run.push_back(Running{clock + N * N * N + 3.0e5, i});
     m->share = (int)std::max<size_t>(1, std::min<size_t>(n, kBatchBytes / m->L.total));
+    int wv[SP_N];
+    std::copy(m->wv, m->wv + SP_N, wv);
+    if (full && m->tuned && !m->fp64 && !m->d.sph)
+      for (int v = 0; v < m->tb->nvariants; ++v)
+        for (int p = 0; p < SP_N; ++p)
+          if (m->tb->staged[v] && m->tb->widths[v] == 8 && ((m->tb->vmask[p] >> v) & 1u)) m->wv[p] = v;
     st = m->fp64 ? do_step<double>(m, 1) : do_step<float>(m, 1);
+    std::copy(wv, wv + SP_N, m->wv);
     if (st == PSC_OK) e = cudaEventRecord(b->events[i + 1], m->st);
   }
   for (int i = 0; i < n && e == cudaSuccess && st == PSC_OK; ++i)
