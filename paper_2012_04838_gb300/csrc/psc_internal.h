@@ -52,8 +52,14 @@ __host__ __device__ constexpr int sphere_storage_halfwidth(int N) {
 // 16-byte multiple, which tensor maps and bulk copies need, whatever M is.  The
 // compact fields keep the pitch M.  Measured at 1024^3 (M = 342, every other row
 // on a half sector): y-inverse 9.69 -> 8.74 ms, y-forward 3.95 -> 3.48 ms; at
-// 512^3 (M = 171) the staged passes it allows: y-inverse 1.55 -> 1.03 ms.
-__host__ __device__ constexpr int row_pitch(int M) { return (M + 3) / 4 * 4; }
+// 512^3 (M = 171) the staged passes it allows: y-inverse 1.55 -> 1.03 ms.  Rows it
+// would lengthen by more than a tenth (3 and 6 values: grids of 8, 12 and 16)
+// keep the pitch M: nothing is staged there, the streams lie in L2 whole, and
+// the padding made the workspace of 16^3 a quarter larger.
+__host__ __device__ constexpr int row_pitch(int M) {
+  const int padded = (M + 3) / 4 * 4;
+  return 10 * (padded - M) > M ? M : padded;
+}
 
 // Retained half-width K: the 2/3 rule (N-1)/3, or the cube that stores the sphere.
 inline Dims make_dims(int N, int sph = 0) {
