@@ -325,7 +325,9 @@ psc_status psc_shell_spectra_noalloc(const void* state, int32_t N, int32_t preci
  * that psc_step() runs for grid size N and precision (2/3 rule), launched
  * nlaunch times over `rows` rows of a deterministic synthetic input instead of
  * the N*N rows of a box, so that hardware-counter captures of it fit in a few
- * GB of device memory.  rows: a positive multiple of 64, at most N*N.  buf:
+ * GB of device memory.  rows: a positive multiple of 64, at most N*N; fewer than
+ * N*N only where the X pass takes a row count (N = 512 and 1024, and N = 256 in
+ * FP32-mixed), PSC_EINVAL elsewhere.  buf:
  * caller-owned device memory of psc_xpass_probe_bytes() bytes, 256-byte
  * aligned, holding a control block, twiddles, the nine input streams
  * [stream][row][kx] and the four output streams; the call fills all but the

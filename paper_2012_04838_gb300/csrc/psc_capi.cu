@@ -1024,6 +1024,10 @@ psc_status probe_check(int32_t N, int32_t precision, int64_t rows) {
   if (precision != PSC_FP64 && precision != PSC_FP32_MIXED) return fail(PSC_EINVAL, "probe: bad precision");
   if (rows <= 0 || rows % 64 != 0 || rows > (int64_t)N * N)
     return fail(PSC_EINVAL, "probe: rows must be a positive multiple of 64, at most N*N");
+  // the register X pass of the other sizes runs N*N rows at their own stride: in
+  // buffers of fewer rows it would read and write past their ends
+  if (rows != (int64_t)N * N && !(precision == PSC_FP64 ? table_f64(N) : table_f32(N))->any_rows)
+    return fail(PSC_EINVAL, "probe: the X pass of this grid size and precision runs N*N rows only");
   return PSC_OK;
 }
 

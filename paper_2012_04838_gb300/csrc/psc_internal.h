@@ -190,6 +190,8 @@ struct PassTable {
   int staged[5];    // 1: input tiles staged through shared memory by TMA
   unsigned vmask[SP_N];  // variants built for each pass (bit v)
   int row_only;  // 1: the X pass exists only as the row X pass (no convective form)
+  int any_rows;  // 1: the right-hand side's X pass takes its rows and stream stride from Dims::ys,
+                 // 0: it always runs N*N rows
 };
 
 const PassTable* table_f32(int N);

@@ -1286,7 +1286,7 @@ template <typename T, int N> struct Passes {
     static const PassTable tb = {&zinv, &yinv, &xpass, &yfwd, &zfwd,
                                  xwarps(), NV,
                                  {WV0, WV1, 4, 8, 16}, {0, 0, 1, 1, 1},
-                                 {MASK_INV, MASK_INV, MASK_FWD, MASK_FWD}, XROW ? 1 : 0};
+                                 {MASK_INV, MASK_INV, MASK_FWD, MASK_FWD}, XROW ? 1 : 0, X2 || X2S ? 1 : 0};
     return &tb;
   }
 };
@@ -1452,7 +1452,7 @@ template <typename T, int N> struct PassesPS {
     static const PassTable tb = {&zinv, &yinv, &xpass, &yfwd, &zfwd,
                                  B::xwarps_unstaged(), NVS,
                                  {WV0, WV1, 4, 8, 16}, {0, 0, 1, 1, 1},
-                                 {MASK_INV, MASK_INV, MASK_FWD, MASK_FWD}, ROWS ? 1 : 0};
+                                 {MASK_INV, MASK_INV, MASK_FWD, MASK_FWD}, ROWS ? 1 : 0, B::X2 || B::X2S ? 1 : 0};
     return &tb;
   }
 };
