@@ -703,7 +703,7 @@ psc_status do_stats(psc_sim* s, double* Ek, double* Ephi, int cap, int* nshell, 
   });
   double* shells = (double*)(s->ws + s->L.shells);
   launch(s, PSC_K_OTHER, 2, [&] {
-    k_reduce_moments<<<NQ, 256, 0, s->st>>>(a.partials, s->tb->xwarps, s->ctrl);
+    k_reduce_moments<<<NQ, 256, 0, s->st>>>(a.partials, s->tb->stat_rows(a), s->ctrl);
     k_shells<T><<<s->nshell * SHELL_PARTS, 256, 0, s->st>>>(d, U, (const unsigned char*)U + 3 * d.S * (s->fp64 ? 16 : 8),
                                                s->nshell, shells);
   });

@@ -136,7 +136,7 @@ struct PassArgs {
   void* yf;         // y-forward output  [4][N][P][MP]  (aliases yb)
   void* rb;         // z-forward output  [4][P][P][M]   compact, unprojected
   const void* tw;   // exp(-2 pi i j/N), j < N
-  double* partials; // X-pass statistics partials [xwarps][NQ]
+  double* partials; // X-pass statistics partials [stat_rows][NQ]
   Ctrl* ctrl;
   int want_umax;    // X pass also reduces max |u1|+|u2|+|u3|
   const void* phase; // exp(i k pi / N), k = -K..K (phase-shift dealiasing)
@@ -184,7 +184,8 @@ struct PassTable {
   void (*xpass)(const PassArgs&, int mode);
   void (*yfwd)(const PassArgs&, int v);
   void (*zfwd)(const PassArgs&, int v);
-  int xwarps;       // warps launched by the X pass (rows of `partials`)
+  int (*stat_rows)(const PassArgs&);  // rows of `partials` that the statistics X pass writes (at most xwarps)
+  int xwarps;       // rows of `partials` that a workspace holds
   int nvariants;    // variants of the strided passes (at most 5)
   int widths[5];    // their column tile widths
   int staged[5];    // 1: input tiles staged through shared memory by TMA

@@ -18,6 +18,7 @@
 // inverse is applied once, to the physical fields in the X pass.
 #pragma once
 
+#include <atomic>
 #include <cstring>
 
 #include "psc_scalars.cuh"
@@ -1048,21 +1049,29 @@ template <typename T, int N> struct Passes {
     const long long cap = 152 * 64;
     return (int)(g < cap ? g : cap);
   }
-  // X-pass CTAs (row X pass) or warps (register X passes) that write statistics partials
-  static int xwarps_unstaged() {
+  // Statistics partials a workspace holds: one row per X-pass CTA (row X pass) or
+  // warp (register X passes).  A constant, the same whatever devices there are and
+  // before any is used: the grid of the staged pass, which follows the device that
+  // it runs on, is kept within it.
+  static int xwarps() {
     if constexpr (XROW) return xrow_grid();
     else return xgrid() * (X2 ? 4 : XW);
   }
-  static int xwarps() {
-    if constexpr (X2S) return xstaged_grid<XMODE_STATS>() * (X2SCfg<T, N, (N - 1) / 3, XMODE_STATS>::THREADS / 32);
-    else return xwarps_unstaged();
+  // rows of partials that the statistics launch of `a` writes
+  static int stat_rows(const PassArgs& a) {
+    if constexpr (X2S) {
+      if (!(XROW_OK && a.xrow))
+        return xstaged_grid<XMODE_STATS>() * (X2SCfg<T, N, (N - 1) / 3, XMODE_STATS>::THREADS / 32);
+    }
+    (void)a;
+    return xwarps();
   }
   // grid: one CTA per statistics partials slot (xwarps()) except where the
   // row X pass is the only one
   template <int MODE, int KK, bool SH> static void xrow_launch(const PassArgs& a) {
     constexpr int WR = XRC::WR;
     using XS = XRowSmem<T, N, WR>;
-    const int grid = XROW ? xrow_grid() : KK == PlanD<N>::K ? xwarps() : xwarps_unstaged();
+    const int grid = XROW ? xrow_grid() : xwarps();
     prep(k_xrow<T, N, WR, MODE, KK, SH>, XS::SMEM);
     launch_kernel(a.pdl != 0, k_xrow<T, N, WR, MODE, KK, SH>, grid, XS::THREADS, XS::SMEM, a.st, a);
   }
@@ -1092,16 +1101,17 @@ template <typename T, int N> struct Passes {
   }
 
   static int sm_count() {
-    static int n[64] = {0};
+    static std::atomic<int> n[64];
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return 152;
-    if (n[dev] == 0) {
-      int c = 0;
+    int c = n[dev].load(std::memory_order_relaxed);
+    if (c == 0) {
       cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev);
-      n[dev] = c > 0 ? c : 152;
+      if (c <= 0) c = 152;
+      n[dev].store(c, std::memory_order_relaxed);
     }
-    return n[dev];
+    return c;
   }
   // Shares (grid z) that the nt transforms of a strided pass are cut into.  A
   // CTA otherwise runs them one after another, which is right where the tiles
@@ -1247,10 +1257,14 @@ template <typename T, int N> struct Passes {
       launch_kernel(a.pdl != 0, k_xpass<T, N, MODE>, xgrid(), 32 * XW, sm, a.st, a);
     }
   }
-  // the staged x pass: one CTA per SM
+  // the staged x pass: one CTA per SM (statistics: no more than have a row of
+  // partials per warp, 405 at 256^3 and 810 at 512^3 and 1024^3)
   template <int MODE> static int xstaged_grid() {
-    const long long rows = (long long)N * N / X2SCfg<T, N, (N - 1) / 3, MODE>::ROWS;
-    return (int)(rows < sm_count() ? rows : sm_count());
+    using SC = X2SCfg<T, N, (N - 1) / 3, MODE>;
+    const long long rows = (long long)N * N / SC::ROWS;
+    int grid = (int)(rows < sm_count() ? rows : sm_count());
+    if (MODE == XMODE_STATS && grid > xwarps() / (SC::THREADS / 32)) grid = xwarps() / (SC::THREADS / 32);
+    return grid;
   }
   template <int MODE> static void xpass_staged(const PassArgs& a) {
     constexpr int KD = (N - 1) / 3;
@@ -1284,7 +1298,7 @@ template <typename T, int N> struct Passes {
   }
   static const PassTable* table() {
     static const PassTable tb = {&zinv, &yinv, &xpass, &yfwd, &zfwd,
-                                 xwarps(), NV,
+                                 &stat_rows, xwarps(), NV,
                                  {WV0, WV1, 4, 8, 16}, {0, 0, 1, 1, 1},
                                  {MASK_INV, MASK_INV, MASK_FWD, MASK_FWD}, XROW ? 1 : 0, X2 || X2S ? 1 : 0};
     return &tb;
@@ -1448,9 +1462,11 @@ template <typename T, int N> struct PassesPS {
       return a.shift ? xpass_k<XMODE_CONVECTIVE, true>(a) : xpass_k<XMODE_CONVECTIVE, false>(a);
     a.shift ? xpass_k<XMODE_RHS, true>(a) : xpass_k<XMODE_RHS, false>(a);
   }
+  // the statistics over the sphere's cube run on the unstaged X passes
+  static int stat_rows(const PassArgs&) { return B::xwarps(); }
   static const PassTable* table() {
     static const PassTable tb = {&zinv, &yinv, &xpass, &yfwd, &zfwd,
-                                 B::xwarps_unstaged(), NVS,
+                                 &stat_rows, B::xwarps(), NVS,
                                  {WV0, WV1, 4, 8, 16}, {0, 0, 1, 1, 1},
                                  {MASK_INV, MASK_INV, MASK_FWD, MASK_FWD}, ROWS ? 1 : 0, B::X2 || B::X2S ? 1 : 0};
     return &tb;
