@@ -107,7 +107,10 @@ __device__ __forceinline__ void b_iftab(int K, const Ctrl* ctrl, double nu, doub
 __device__ __forceinline__ void b_cfl(Ctrl* c, double cfl, double dx, int record_every) {
   if (c->step % record_every != 0) return;
   const double m = __longlong_as_double((long long)c->umax_bits);
-  if (!(m <= 1.7976931348623157e308)) { c->err |= 2; return; }
+  if (!(m <= 1.7976931348623157e308)) {
+    atomicOr(&c->err, 2);  // beside CTAs that may be raising, or polling, the time-out bit
+    return;
+  }
   if (m > 0.0) c->dt = cfl * dx / m;
 }
 
