@@ -93,9 +93,6 @@ template <int N> struct PlanD : Plan<N> {
   static_assert(32 % TPL == 0, "a line's threads must sit inside one warp");
 };
 
-// FP64 lines whose second step, of size R, takes its twiddles in (dft_tw)
-template <typename T, int N, int R> constexpr bool kTwRead = sizeof(T) == 8 && (R == 4 || R == 8 || R == 16);
-
 // Programmatic dependent launch: a pass is launched while the one before it in
 // the stream drains (launch_kernel), so its CTAs start, and fill their twiddle
 // tables, beside the last CTAs of that pass.  pdl_wait() returns once every

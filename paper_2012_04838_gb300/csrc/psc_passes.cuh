@@ -67,8 +67,8 @@ __device__ __forceinline__ typename CT<T>::type* strided_twiddles(unsigned char*
   C* t = reinterpret_cast<C*>(smraw + StridedSmem<T, N, W>::EXCH_BYTES);
   const int nthr = tcx.bdx * tcx.bdy, me = tcx.ty * tcx.bdx + tcx.tx;
   for (int i = me; i < N; i += nthr) {
-    if constexpr (PL::WIDE || kTwRead<T, N, PL::R2>) {
-      t[i] = tw[i];  // indexed by the exponent
+    if constexpr (PL::WIDE) {
+      t[i] = tw[i];  // wide lines index wN^(n2 k1) directly
     } else {
       const int tt = i % PL::TPL, k1 = (i / PL::TPL) % PL::R1, j = i / (PL::TPL * PL::R1);
       t[i] = tw[(tt + j * PL::TPL) * k1];
@@ -113,71 +113,6 @@ template <int N, int KK = (N - 1) / 3> __host__ __device__ constexpr bool dead_k
   return PlanD<N>::R1 * k2 > KK && PlanD<N>::R1 * k2 + PlanD<N>::R1 - 1 < N - KK;
 }
 
-// DFT of size R (4, 8 or 16) of x[n] w^n, w = wN^q: the second step of a line
-// with its twiddles taken in, as radix-4 and radix-2 butterflies a +- w b of six
-// fused multiply-adds each (the difference is 2 a minus the sum; Linzer and Feig
-// 1993 give such forms).  The 15 products and the DFT-16 after them are 220
-// operations, this is 192, and FP64 is bound by their number (the pipe was 86%
-// busy): at 256^3 the X pass went from 5.77 to 5.32 ms a launch, the y-inverse from
-// 2.30 to 2.11.  wt(e) is wN^e (forward sign), e < N.
-template <int DIR, class C> __device__ __forceinline__ void bfly(C& a, C& b, C w) {
-  if (DIR > 0) w.y = -w.y;
-  const C s = mk(fma(-w.y, b.y, fma(w.x, b.x, a.x)), fma(w.y, b.x, fma(w.x, b.y, a.y)));
-  b = mk(fma(2.0, a.x, -s.x), fma(2.0, a.y, -s.y));
-  a = s;
-}
-// a, b <- a + r w b, a - r w b with r = i DIR
-template <int DIR, class C> __device__ __forceinline__ void bfly_i(C& a, C& b, C w) {
-  if (DIR > 0) w.y = -w.y;
-  C s;
-  if (DIR < 0) s = mk(fma(w.y, b.x, fma(w.x, b.y, a.x)), fma(w.y, b.y, fma(-w.x, b.x, a.y)));
-  else s = mk(fma(-w.y, b.x, fma(-w.x, b.y, a.x)), fma(-w.y, b.y, fma(w.x, b.x, a.y)));
-  b = mk(fma(2.0, a.x, -s.x), fma(2.0, a.y, -s.y));
-  a = s;
-}
-// DFT-4 of (a, w b, w^2 c, w^3 d), outputs in a, b, c, d
-template <int DIR, class C> __device__ __forceinline__ void dft4_tw(C& a, C& b, C& c, C& d, C w, C w2) {
-  bfly<DIR>(a, c, w2);
-  bfly<DIR>(b, d, w2);     // w b +- w^3 d = w (b +- w^2 d)
-  bfly<DIR>(a, b, w);      // a: X0, b: X2
-  bfly_i<DIR>(c, d, w);    // c: X1, d: X3
-  const C x2 = b;
-  b = c;
-  c = x2;
-}
-template <int N, int R, int DIR, class C, class WT>
-__device__ __forceinline__ void dft_tw(C (&x)[R], int q, const WT& wt) {
-  if constexpr (R == 4) {
-    dft4_tw<DIR>(x[0], x[1], x[2], x[3], wt(q), wt(2 * q));
-  } else if constexpr (R == 8) {
-    // X[k + 4 m] = sum_r (-1)^(r m) (w w8^k)^r sum_j w4^(j k) w^(2 j) x[r + 2 j]
-    const C al = wt(2 * q), al2 = wt(4 * q);
-    dft4_tw<DIR>(x[0], x[2], x[4], x[6], al, al2);
-    dft4_tw<DIR>(x[1], x[3], x[5], x[7], al, al2);
-    // x[2 k + r] holds the inner sum of (r, k)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) bfly<DIR>(x[2 * k], x[2 * k + 1], wt(q + k * (N / 8)));
-    const C y[8] = {x[0], x[2], x[4], x[6], x[1], x[3], x[5], x[7]};
-#pragma unroll
-    for (int k = 0; k < 8; ++k) x[k] = y[k];
-  } else {
-    // X[k + 4 m] = sum_r w4^(r m) (w w16^k)^r sum_j w4^(j k) w^(4 j) x[r + 4 j]
-    const C al = wt(4 * q), al2 = wt(8 * q);
-#pragma unroll
-    for (int r = 0; r < 4; ++r) dft4_tw<DIR>(x[r], x[r + 4], x[r + 8], x[r + 12], al, al2);
-    // x[r + 4 k] holds the inner sum of (r, k)
-    C y[16];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      dft4_tw<DIR>(x[4 * k], x[4 * k + 1], x[4 * k + 2], x[4 * k + 3], wt(q + k * (N / 16)), wt(2 * q + k * (N / 8)));
-#pragma unroll
-      for (int m = 0; m < 4; ++m) y[k + 4 * m] = x[4 * k + m];
-    }
-#pragma unroll
-    for (int k = 0; k < 16; ++k) x[k] = y[k];
-  }
-}
-
 // One length-N DFT per column, direction DIR (-1 forward, +1 inverse).
 // ld(p) returns the element at line position p; st(k, v) stores output k.
 // A forward transform only computes the outputs a truncated pass can keep.
@@ -202,7 +137,7 @@ __device__ __forceinline__ void strided_fft(const LD& ld, const ST& st,
 #pragma unroll
     for (int k1 = 0; k1 < R1; ++k1) {
       C v = a[k1];
-      if (k1 > 0 && !kTwRead<T, N, R2>) {
+      if (k1 > 0) {
         const C wv = twsm[(j * R1 + k1) * TPL + t];  // wN^(n2 k1)
         v = (DIR < 0) ? cmul(v, wv) : cmulc(v, wv);
       }
@@ -214,8 +149,7 @@ __device__ __forceinline__ void strided_fft(const LD& ld, const ST& st,
     C b[R2];
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) b[n2] = sm[k1 * SM::ROW + n2 * W + w];
-    if constexpr (!PL::WIDE && kTwRead<T, N, R2>) dft_tw<N, R2, DIR>(b, k1, [&](int e) { return twsm[e]; });
-    else Dft<R2, DIR>::template run<T, C>(b);
+    Dft<R2, DIR>::template run<T, C>(b);
     static_for<0, R2>([&](auto kc) {
       constexpr int k2 = decltype(kc)::value;
       if constexpr (!(DIR < 0 && dead_k2<N, KK>(k2))) st(k1 + R1 * k2, b[k2]);
@@ -587,7 +521,7 @@ __device__ __forceinline__ void xinv(const SPEC& spec,
 #pragma unroll
     for (int k1 = 0; k1 < R1; ++k1) {
       C v = a[k1];
-      if (k1 > 0 && !kTwRead<T, N, R2>) v = cmulc(v, tw[(j * R1 + k1) * TPL + t]);  // wN^(-n2 k1)
+      if (k1 > 0) v = cmulc(v, tw[(j * R1 + k1) * TPL + t]);  // wN^(-n2 k1)
       ex[k1 * XC::ROWI + n2] = v;
     }
   });
@@ -597,8 +531,7 @@ __device__ __forceinline__ void xinv(const SPEC& spec,
     const int k1 = t + j * TPL;
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) z[j][n2] = ex[k1 * XC::ROWI + n2];
-    if constexpr (kTwRead<T, N, R2>) dft_tw<N, R2, +1>(z[j], k1, [&](int e) { return tw[e]; });
-    else Dft<R2, +1>::template run<T, C>(z[j]);
+    Dft<R2, +1>::template run<T, C>(z[j]);
     if constexpr (SCALE) {
 #pragma unroll
       for (int k2 = 0; k2 < R2; ++k2) z[j][k2] = cscale(z[j][k2], scale);
@@ -627,7 +560,7 @@ __device__ __forceinline__ void xfwd(typename CT<T>::type (&x)[PlanD<N>::J2][Pla
 #pragma unroll
     for (int k1 = 0; k1 < R2; ++k1) {
       C v = x[j][k1];
-      if (k1 > 0 && !kTwRead<T, N, R1>) v = cmul(v, tw[N + (j * R2 + k1) * TPL + t]);  // wN^(n2 k1)
+      if (k1 > 0) v = cmul(v, tw[N + (j * R2 + k1) * TPL + t]);  // wN^(n2 k1)
       ex[k1 * XC::ROWF + n2] = v;
     }
   }
@@ -638,8 +571,7 @@ __device__ __forceinline__ void xfwd(typename CT<T>::type (&x)[PlanD<N>::J2][Pla
     const int k1 = t + j * TPL;
 #pragma unroll
     for (int n2 = 0; n2 < R1; ++n2) b[j][n2] = ex[k1 * XC::ROWF + n2];
-    if constexpr (kTwRead<T, N, R1>) dft_tw<N, R1, -1>(b[j], k1, [&](int e) { return tw[N + e]; });
-    else Dft<R1, -1>::template run<T, C>(b[j]);
+    Dft<R1, -1>::template run<T, C>(b[j]);
   }
   __syncwarp();
   static_for<0, PL::J1>([&](auto jc) {
@@ -685,9 +617,9 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
     for (int i = tcx.tx; i < N; i += tcx.bdx) {
       const int tt = i % TPL;
       const int k1i = (i / TPL) % R1, ji = i / (TPL * R1);  // inverse: k1 < R1, j < J1
-      tw[i] = twg[kTwRead<T, N, R2> ? i : (tt + ji * TPL) * k1i];
+      tw[i] = twg[(tt + ji * TPL) * k1i];
       const int k1f = (i / TPL) % R2, jf = i / (TPL * R2);  // forward: k1 < R2, j < J2
-      tw[N + i] = twg[kTwRead<T, N, R1> ? i : (tt + jf * TPL) * k1f];
+      tw[N + i] = twg[(tt + jf * TPL) * k1f];
     }
     __syncthreads();
   }
