@@ -479,6 +479,7 @@ __device__ __forceinline__ void xinv(const SPEC& spec,
                                      typename CT<T>::type* ex,
                                      const typename CT<T>::type* tw, int t, T scale,
                                      const void* phase = nullptr) {
+  static_assert(SCALE || !kScaled<T, N>, "the inverse table carries the scale");
   using C = typename CT<T>::type;
   using PL = PlanD<N>;
   using XC = XCfg<T, N>;
@@ -521,7 +522,8 @@ __device__ __forceinline__ void xinv(const SPEC& spec,
 #pragma unroll
     for (int k1 = 0; k1 < R1; ++k1) {
       C v = a[k1];
-      if (k1 > 0) v = cmulc(v, tw[(j * R1 + k1) * TPL + t]);  // wN^(-n2 k1)
+      if (k1 > 0) v = cmulc(v, tw[(j * R1 + k1) * TPL + t]);  // wN^(-n2 k1), times 1/N^3 where kScaled
+      else if constexpr (kScaled<T, N>) v = cscale(v, scale);
       ex[k1 * XC::ROWI + n2] = v;
     }
   });
@@ -532,7 +534,7 @@ __device__ __forceinline__ void xinv(const SPEC& spec,
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) z[j][n2] = ex[k1 * XC::ROWI + n2];
     Dft<R2, +1>::template run<T, C>(z[j]);
-    if constexpr (SCALE) {
+    if constexpr (SCALE && !kScaled<T, N>) {
 #pragma unroll
       for (int k2 = 0; k2 < R2; ++k2) z[j][k2] = cscale(z[j][k2], scale);
     }
@@ -612,12 +614,14 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
   const C* PSC_RESTRICT yb = static_cast<const C*>(a.yb);
   C* PSC_RESTRICT xb = static_cast<C*>(a.xb);
   C* tw = reinterpret_cast<C*>(smraw + XC::LINE_BYTES * LPW * XW);
+  const T scale = T(1.0 / ((double)N * N * N));
   {
     const C* PSC_RESTRICT twg = static_cast<const C*>(a.tw);
     for (int i = tcx.tx; i < N; i += tcx.bdx) {
       const int tt = i % TPL;
       const int k1i = (i / TPL) % R1, ji = i / (TPL * R1);  // inverse: k1 < R1, j < J1
-      tw[i] = twg[(tt + ji * TPL) * k1i];
+      const C w = twg[(tt + ji * TPL) * k1i];
+      tw[i] = kScaled<T, N> ? cscale(w, scale) : w;
       const int k1f = (i / TPL) % R2, jf = i / (TPL * R2);  // forward: k1 < R2, j < J2
       tw[N + i] = twg[(tt + jf * TPL) * k1f];
     }
@@ -628,13 +632,13 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
   constexpr long long nlines = (long long)N * N;
   // every group of a warp is full: no row needs a bounds test
   constexpr bool FULL = nlines % LPW == 0;
-  const T scale = T(1.0 / ((double)N * N * N));
-  // the inverse transforms of the right-hand side are left unscaled (N^3 times
-  // the fields); each product carries the missing 1/N^6 once
-  const T s2 = scale * scale;
+  // unless SC, the inverse transforms of the right-hand side are left unscaled (N^3
+  // times the fields) and each product carries the missing 1/N^6 once
+  constexpr bool SC = kScaled<T, N>;
+  const T s2 = SC ? T(1) : scale * scale;
   const C zero = mk(T(0), T(0));
-  // maximum of |u1|+|u2|+|u3| over the thread's points (unscaled fields in the
-  // right-hand side, scaled in the statistics)
+  // maximum of |u1|+|u2|+|u3| over the thread's points (of the fields as the mode
+  // forms them: scaled in the statistics)
   T um = T(0);
   MomentSum<T> acc[MODE == XMODE_STATS ? NQ : 1];
 
@@ -672,7 +676,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
         else return c == 0 ? ux[j][k2] : (c == 1 ? uy[j][k2] : uz[j][k2]);
       };
       // (u1, u2)
-      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UY, kx); }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UY, kx); }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
@@ -686,7 +690,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
           }
         }
       // (u3, omega_1)
-      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UZ, kx); x2 = Y(Y_WX, kx); }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UZ, kx); x2 = Y(Y_WX, kx); }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
@@ -698,7 +702,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
           if (a.want_umax) um = max_keep_nan(um, fabs(getu(0, j, k2)) + fabs(getu(1, j, k2)) + fabs(u3));
         }
       // (omega_2, omega_3):  omega_2 = d_z u_1 - i kx u_3,  omega_3 = i kx u_2 - d_y u_1
-      xinv<T, N, false, KK, SHIFT>(
+      xinv<T, N, SC, KK, SHIFT>(
           [&](int kx, C& x1, C& x2) {
             x1 = csub(Y(Y_DZUX, kx), mul_ik(Y(Y_UZ, kx), T(kx)));
             x2 = csub(mul_ik(Y(Y_UY, kx), T(kx)), Y(Y_DYUX, kx));
@@ -727,7 +731,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
         continue;
       }
       // (dphi/dx1, dphi/dx2); the slot of u1 then holds the partial u . grad phi
-      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); },
+      xinv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); },
                  z, ex, tw, t, scale, a.phase);
       T sv[J2][R2];
 #pragma unroll
@@ -736,7 +740,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
         for (int k2 = 0; k2 < R2; ++k2)
           sv[j][k2] = dot2(getu(0, j, k2), z[j][k2].x, getu(1, j, k2), z[j][k2].y);
       // (dphi/dx3, 0)
-      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
@@ -761,13 +765,13 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
         }
       };
       // (u1, u2)
-      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UY, kx); }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UY, kx); }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) { putu(0, j, k2, z[j][k2].x); putu(1, j, k2, z[j][k2].y); }
       // (u3, d1 u1)
-      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UZ, kx); x2 = mul_ik(Y(Y_UX, kx), T(kx)); }, z, ex, tw, t,
+      xinv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UZ, kx); x2 = mul_ik(Y(Y_UX, kx), T(kx)); }, z, ex, tw, t,
                  scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
@@ -778,20 +782,20 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
           if (a.want_umax) um = max_keep_nan(um, fabs(getu(0, j, k2)) + fabs(getu(1, j, k2)) + fabs(z[j][k2].x));
         }
       // (d2 u1, d3 u1): aa = (u.grad) u1
-      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DYUX, kx); x2 = Y(Y_DZUX, kx); }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DYUX, kx); x2 = Y(Y_DZUX, kx); }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) aa[j][k2] += getu(1, j, k2) * z[j][k2].x + getu(2, j, k2) * z[j][k2].y;
       // (d1 u2, d2 u2)
-      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_UY, kx), T(kx)); x2 = Y(Y_DYUY, kx); }, z, ex, tw, t,
+      xinv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_UY, kx), T(kx)); x2 = Y(Y_DYUY, kx); }, z, ex, tw, t,
                  scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) bb[j][k2] = getu(0, j, k2) * z[j][k2].x + getu(1, j, k2) * z[j][k2].y;
       // (d3 u2, d1 u3): bb = (u.grad) u2; aa starts (u.grad) u3
-      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZUY, kx); x2 = mul_ik(Y(Y_UZ, kx), T(kx)); }, z, ex, tw, t,
+      xinv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZUY, kx); x2 = mul_ik(Y(Y_UZ, kx), T(kx)); }, z, ex, tw, t,
                  scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
@@ -803,20 +807,20 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
         }
       xfwd<T, N, KK, SHIFT>(z, store(0), ex, tw, t, a.phase);
       // (d2 u3, d3 u3): aa = (u.grad) u3
-      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_WX, kx); x2 = Y(Y_DZUZ, kx); }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_WX, kx); x2 = Y(Y_DZUZ, kx); }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) aa[j][k2] += getu(1, j, k2) * z[j][k2].x + getu(2, j, k2) * z[j][k2].y;
       // (dphi/dx1, dphi/dx2)
-      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); }, z, ex, tw, t,
+      xinv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); }, z, ex, tw, t,
                  scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
         for (int k2 = 0; k2 < R2; ++k2) bb[j][k2] = getu(0, j, k2) * z[j][k2].x + getu(1, j, k2) * z[j][k2].y;
       // (dphi/dx3, 0)
-      xinv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, tw, t, scale, a.phase);
+      xinv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, tw, t, scale, a.phase);
 #pragma unroll
       for (int j = 0; j < J2; ++j)
 #pragma unroll
@@ -903,7 +907,7 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
   }
 
   if (MODE == XMODE_STATS || a.want_umax) {
-    double umax = MODE == XMODE_STATS ? (double)um : (double)um * (double)scale;
+    double umax = MODE == XMODE_STATS || SC ? (double)um : (double)um * (double)scale;
     for (int o = 16; o > 0; o >>= 1) {
       const double other = __shfl_xor_sync(0xffffffffu, umax, o);
       umax = other > umax || other != other ? other : umax;

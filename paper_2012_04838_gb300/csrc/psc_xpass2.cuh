@@ -167,6 +167,7 @@ template <typename T, int N, bool SCALE = true, int KK = (N - 1) / 3, bool SHIFT
 __device__ __forceinline__ void x2inv(const SPEC& spec, typename CT<T>::type (&z)[16],
                                       typename CT<T>::type* ex, const X2Roles<typename CT<T>::type>& q,
                                       T scale, const void* phase = nullptr) {
+  static_assert(SCALE || !kScaled<T, N>, "the inverse table carries the scale");
   using C = typename CT<T>::type;
   using XC = X2Cfg<T, N>;
   constexpr int TH = XC::TH, G = XC::G, ROW = XC::ROW, K = KK;
@@ -212,7 +213,8 @@ __device__ __forceinline__ void x2inv(const SPEC& spec, typename CT<T>::type (&z
   for (int a = 0; a < 16; a += 2) {
     C w0, w1;
     tw_pair<T, TH>(q.t1, a, q.tid, w0, w1);
-    const C u0 = a > 0 ? cmulc(v[a], w0) : v[a];  // wN^(-a j)
+    // wN^(-a j), times 1/N^3 where kScaled
+    const C u0 = a > 0 ? cmulc(v[a], w0) : kScaled<T, N> ? cscale(v[a], scale) : v[a];
     ex[a * ROW + q.tid] = u0;
     ex[(a + 1) * ROW + q.tid] = cmulc(v[a + 1], w1);
   }
@@ -231,7 +233,7 @@ __device__ __forceinline__ void x2inv(const SPEC& spec, typename CT<T>::type (&z
     }
   }
   lane_dft<T, G, +1>(z, q.rr);  // over k0 -> c
-  if constexpr (SCALE) {
+  if constexpr (SCALE && !kScaled<T, N>) {
 #pragma unroll
     for (int b = 0; b < 16; ++b) z[b] = cscale(z[b], scale);
   }
@@ -303,7 +305,7 @@ __device__ __forceinline__ void x2_twiddles(typename CT<T>::type* t1, const type
   for (int i = threadIdx.x; i < 16 * TH; i += blockDim.x) {
     const int e = i / TH, tid = i % TH;  // e = a for T1, k1 for T3
     const int ra = tid / G, rk0 = bitrev_lane<G>(tid % G);
-    t1[tw_index<T, TH>(e, tid)] = tw[e * tid];
+    t1[tw_index<T, TH>(e, tid)] = kScaled<T, N> ? cscale(tw[e * tid], T(1.0 / ((double)N * N * N))) : tw[e * tid];
     t3[tw_index<T, TH>(e, tid)] = tw[ra * (rk0 + G * e)];
   }
   for (int i = threadIdx.x; i < 16 * G; i += blockDim.x) t2[tw_index<T, G>(i / G, i % G)] = tw[16 * (i / G) * (i % G)];
@@ -330,17 +332,18 @@ __device__ __forceinline__ bool x2_rhs_row(const YF& Y, const HA& after_a, const
   const C zero = mk(T(0), T(0));
   (void)ctrl;
   C z[16];
-  // the inverse transforms are left unscaled (N^3 times the fields); each
-  // product carries the missing 1/N^6 once
-  const T s2 = scale * scale;
+  // unless SC, the inverse transforms are left unscaled (N^3 times the fields) and
+  // each product carries the missing 1/N^6 once
+  constexpr bool SC = kScaled<T, N>;
+  const T s2 = SC ? T(1) : scale * scale;
   // live per thread at most: u1, u2, u3 and one more field (64 values)
   T u1[16], u2[16], u3[16], W[16];
   // (u1, u2)
-  x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UY, kx); }, z, ex, q, scale, phase);
+  x2inv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UY, kx); }, z, ex, q, scale, phase);
 #pragma unroll
   for (int b = 0; b < 16; ++b) { u1[b] = z[b].x; u2[b] = z[b].y; }
   // (u3, omega1)
-  x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UZ, kx); x2 = Y(Y_WX, kx); }, z, ex, q, scale, phase);
+  x2inv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UZ, kx); x2 = Y(Y_WX, kx); }, z, ex, q, scale, phase);
 #pragma unroll
   for (int b = 0; b < 16; ++b) {
     u3[b] = z[b].x;
@@ -348,7 +351,7 @@ __device__ __forceinline__ bool x2_rhs_row(const YF& Y, const HA& after_a, const
     if (want_umax) um = max_keep_nan(um, fabs(u1[b]) + fabs(u2[b]) + fabs(u3[b]));
   }
   // (omega2, omega3): omega2 = d_z u1 - i kx u3, omega3 = i kx u2 - d_y u1
-  x2inv<T, N, false, KK, SHIFT>(
+  x2inv<T, N, SC, KK, SHIFT>(
       [&](int kx, C& x1, C& x2) {
         x1 = csub(Y(Y_DZUX, kx), mul_ik(Y(Y_UZ, kx), T(kx)));
         x2 = csub(mul_ik(Y(Y_UY, kx), T(kx)), Y(Y_DYUX, kx));
@@ -382,12 +385,12 @@ __device__ __forceinline__ bool x2_rhs_row(const YF& Y, const HA& after_a, const
   }
   if (!wait_b()) return false;
   // (dphi/dx1, dphi/dx2); u1 then holds the partial u . grad phi
-  x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); },
+  x2inv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); },
                      z, ex, q, scale, phase);
 #pragma unroll
   for (int b = 0; b < 16; ++b) u1[b] = dot2(u1[b], z[b].x, u2[b], z[b].y);
   // (dphi/dx3, 0)
-  x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, q, scale, phase);
+  x2inv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, q, scale, phase);
   after_b();
 #pragma unroll
   for (int b = 0; b < 16; ++b) z[b] = mk(W[b] * s2, fma(u3[b], z[b].x, u1[b]) * s2);  // (NL3, u.grad phi)
@@ -418,7 +421,8 @@ __device__ __forceinline__ bool x2_conv_row(const YF& Y, const HA& after_a, cons
   const C zero = mk(T(0), T(0));
   (void)ctrl;
   C z[16];
-  const T s2 = scale * scale;  // the transforms are unscaled: each product carries 1/N^6
+  constexpr bool SC = kScaled<T, N>;
+  const T s2 = SC ? T(1) : scale * scale;  // as in x2_rhs_row
   T u1[16], u2[16], u3[16], A[16], B[16];
   auto out = [&](int s0) {
     return [&, s0](int kx, C X1, C X2) {
@@ -427,11 +431,11 @@ __device__ __forceinline__ bool x2_conv_row(const YF& Y, const HA& after_a, cons
     };
   };
   // (u1, u2)
-  x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UY, kx); }, z, ex, q, scale, phase);
+  x2inv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UY, kx); }, z, ex, q, scale, phase);
 #pragma unroll
   for (int b = 0; b < 16; ++b) { u1[b] = z[b].x; u2[b] = z[b].y; }
   // (u3, d1 u1)
-  x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UZ, kx); x2 = mul_ik(Y(Y_UX, kx), T(kx)); }, z, ex, q,
+  x2inv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UZ, kx); x2 = mul_ik(Y(Y_UX, kx), T(kx)); }, z, ex, q,
                      scale, phase);
 #pragma unroll
   for (int b = 0; b < 16; ++b) {
@@ -440,16 +444,16 @@ __device__ __forceinline__ bool x2_conv_row(const YF& Y, const HA& after_a, cons
     if (want_umax) um = max_keep_nan(um, fabs(u1[b]) + fabs(u2[b]) + fabs(u3[b]));
   }
   // (d2 u1, d3 u1): A = (u.grad) u1
-  x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DYUX, kx); x2 = Y(Y_DZUX, kx); }, z, ex, q, scale, phase);
+  x2inv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DYUX, kx); x2 = Y(Y_DZUX, kx); }, z, ex, q, scale, phase);
 #pragma unroll
   for (int b = 0; b < 16; ++b) A[b] += u2[b] * z[b].x + u3[b] * z[b].y;
   // (d1 u2, d2 u2)
-  x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_UY, kx), T(kx)); x2 = Y(Y_DYUY, kx); }, z, ex, q,
+  x2inv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_UY, kx), T(kx)); x2 = Y(Y_DYUY, kx); }, z, ex, q,
                      scale, phase);
 #pragma unroll
   for (int b = 0; b < 16; ++b) B[b] = u1[b] * z[b].x + u2[b] * z[b].y;
   // (d3 u2, d1 u3): B = (u.grad) u2; A starts (u.grad) u3
-  x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZUY, kx); x2 = mul_ik(Y(Y_UZ, kx), T(kx)); }, z, ex, q,
+  x2inv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZUY, kx); x2 = mul_ik(Y(Y_UZ, kx), T(kx)); }, z, ex, q,
                      scale, phase);
   after_a();
 #pragma unroll
@@ -461,16 +465,16 @@ __device__ __forceinline__ bool x2_conv_row(const YF& Y, const HA& after_a, cons
   x2fwd<T, N, KK, SHIFT>(z, out(0), ex, q, phase);
   if (!wait_b()) return false;
   // (d2 u3, d3 u3): A = (u.grad) u3
-  x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_WX, kx); x2 = Y(Y_DZUZ, kx); }, z, ex, q, scale, phase);
+  x2inv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_WX, kx); x2 = Y(Y_DZUZ, kx); }, z, ex, q, scale, phase);
 #pragma unroll
   for (int b = 0; b < 16; ++b) A[b] += u2[b] * z[b].x + u3[b] * z[b].y;
   // (dphi/dx1, dphi/dx2)
-  x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); }, z, ex,
+  x2inv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_PHI, kx), T(kx)); x2 = Y(Y_DYPHI, kx); }, z, ex,
                      q, scale, phase);
 #pragma unroll
   for (int b = 0; b < 16; ++b) B[b] = u1[b] * z[b].x + u2[b] * z[b].y;
   // (dphi/dx3, 0)
-  x2inv<T, N, false, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, q, scale, phase);
+  x2inv<T, N, SC, KK, SHIFT>([&](int kx, C& x1, C& x2) { x1 = Y(Y_DZPHI, kx); x2 = zero; }, z, ex, q, scale, phase);
   after_b();
 #pragma unroll
   for (int b = 0; b < 16; ++b) z[b] = mk(-A[b] * s2, (B[b] + u3[b] * z[b].x) * s2);  // (NL3, u.grad phi)
@@ -600,8 +604,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : PSC_X2_MINB) k_xpass
   const long long nlines = ys / MP;
   const T scale = T(1.0 / ((double)N * N * N));
   const C zero = mk(T(0), T(0));
-  // maximum of |u1|+|u2|+|u3| over the thread's points (unscaled fields in the
-  // RHS variant, scaled in the statistics variant)
+  // maximum of |u1|+|u2|+|u3| over the thread's points (of the fields as the mode
+  // forms them: scaled in the statistics)
   T um = T(0);
   MomentSum<T> acc[MODE == XMODE_STATS ? NQ : 1];
 
@@ -627,7 +631,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : PSC_X2_MINB) k_xpass
   if (MODE == XMODE_STATS || a.want_umax) {
     // the same value as taking the FP64 maximum point by point: conversion and
     // the positive scaling are monotone
-    double umax = MODE == XMODE_STATS ? (double)um : (double)um * (double)scale;
+    double umax = MODE == XMODE_STATS || kScaled<T, N> ? (double)um : (double)um * (double)scale;
     for (int o = 16; o > 0; o >>= 1) {
       const double other = __shfl_xor_sync(0xffffffffu, umax, o);
       umax = other > umax || other != other ? other : umax;
@@ -852,7 +856,7 @@ __global__ void __launch_bounds__(X2SCfg<T, N, KK, MODE>::THREADS, 1) k_xpass2s(
     }
   }
   if (MODE == XMODE_STATS || a.want_umax) {
-    double umax = MODE == XMODE_STATS ? (double)um : (double)um * (double)scale;
+    double umax = MODE == XMODE_STATS || kScaled<T, N> ? (double)um : (double)um * (double)scale;
     for (int o = 16; o > 0; o >>= 1) {
       const double other = __shfl_xor_sync(0xffffffffu, umax, o);
       umax = other > umax || other != other ? other : umax;
