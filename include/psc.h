@@ -114,8 +114,10 @@ typedef struct {
  * PSC_FP32_MIXED each thread first accumulates its share in compensated FP32
  * (the shell sums behind E(n), K, eps, chi, phi_var, phi_prod, E_forced; the
  * grid moments behind K_phys, eps_phys, chi_phys, phi_prod_phys, skew, flat,
- * skew_phi, flat_phi), which keeps these fields within 2e-5 relative of the
- * FP64 values (skewness and flatness within 1e-4 absolute; tested). */
+ * skew_phi, flat_phi; at N = 512 and 1024 the moments' terms join those sums
+ * sixteen at a time, added up plainly), which keeps these fields within 2e-5
+ * relative of the FP64 values (skewness and flatness within 1e-4 absolute;
+ * tested). */
 typedef struct {
   double t, dt;
   double K, K_phys, eps, eps_phys, eta, Re_lambda, Te, urms, lambda, l0;

@@ -829,11 +829,8 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
       xfwd<T, N, KK, SHIFT>(z, store(2), ex, tw, t, a.phase);
     } else {
       // statistics: moments of the diagonal velocity gradients and the scalar
-      // gradient (Eqs. 11-12), |omega|^2, u.u, phi u2, phi^2 (Eq. 13).  The
-      // thread's points of one field are added up first, in four short chains,
-      // and join the compensated sum once per field and row: a compensated add
-      // per point is four dependent operations for each of 20 sums (the pass
-      // took 108 us at 128^3 against 38 us for the right-hand side).
+      // gradient (Eqs. 11-12), |omega|^2, u.u, phi u2, phi^2 (Eq. 13), each point
+      // added to its compensated sum
       constexpr int NP = J2 * R2;
       T s13[NP], f1[NP], f2[NP];
       auto split = [&]() {
@@ -842,12 +839,9 @@ __device__ __forceinline__ void b_xpass(const PassArgs& a, const Tctx& tcx) {
 #pragma unroll
           for (int k2 = 0; k2 < R2; ++k2) { f1[j * R2 + k2] = z[j][k2].x; f2[j * R2 + k2] = z[j][k2].y; }
       };
-      // acc[q] += sum over the points of term(i)
       auto put = [&](int q, auto&& term) {
-        T s[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
-        for (int i = 0; i < NP; ++i) s[i & 3] += term(i);
-        acc[q].add((s[0] + s[1]) + (s[2] + s[3]));
+        for (int i = 0; i < NP; ++i) acc[q].add(term(i));
       };
       auto mom3 = [&](int q, const T (&f)[NP]) {
         put(q, [&](int i) { return f[i] * f[i]; });

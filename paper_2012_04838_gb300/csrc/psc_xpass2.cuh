@@ -482,8 +482,10 @@ __device__ __forceinline__ bool x2_conv_row(const YF& Y, const HA& after_a, cons
   return true;
 }
 
-// The statistics of one row (Eqs. 11-13): each pair's moments over the thread's 16
-// points are added up plainly and join the thread's compensated sums.  The hooks
+// The statistics of one row (Eqs. 11-13).  EACH: every point joins the thread's
+// compensated sums by itself, as on the grids of the register pass; else (512 and
+// 1024) each pair's moments over the thread's 16 points are added up plainly first,
+// which leaves an error of up to 15 roundings of FP32 in each such sum.  The hooks
 // as in x2_rhs_row: after_a() once all streams but DYPHI, DZPHI and DZUZ are no
 // longer read, wait_b() before those are, after_b() once they are not.
 template <typename T, int N, int KK, class YF, class HA, class WB, class HB>
@@ -493,48 +495,45 @@ __device__ __forceinline__ bool x2_stats_row(const YF& Y, const HA& after_a, con
   using C = typename CT<T>::type;
   const C zero = mk(T(0), T(0));
   C z[16];
+  constexpr bool EACH = N < 512;
   T s13[16];
-  auto mom3 = [&](int slot, auto&& f) {
-    T m2 = T(0), m3 = T(0), m4 = T(0);
+  // acc[slot] takes f(b) of the 16 points
+  auto put = [&](int slot, auto&& f) {
+    if constexpr (EACH) {
 #pragma unroll
-    for (int b = 0; b < 16; ++b) { const T v = f(b), v2 = v * v; m2 += v2; m3 += v2 * v; m4 += v2 * v2; }
-    acc[slot].add(m2);
-    acc[slot + 1].add(m3);
-    acc[slot + 2].add(m4);
+      for (int b = 0; b < 16; ++b) acc[slot].add(f(b));
+    } else {
+      T s = T(0);
+#pragma unroll
+      for (int b = 0; b < 16; ++b) s += f(b);
+      acc[slot].add(s);
+    }
+  };
+  auto mom3 = [&](int slot, auto&& f) {
+    put(slot, [&](int b) { const T v = f(b); return v * v; });
+    put(slot + 1, [&](int b) { const T v = f(b); return v * v * v; });
+    put(slot + 2, [&](int b) { const T v = f(b), v2 = v * v; return v2 * v2; });
   };
   auto re = [&](int b) { return z[b].x; };
   auto im = [&](int b) { return z[b].y; };
+  auto sq2 = [&](int b) { return z[b].x * z[b].x + z[b].y * z[b].y; };
   // (u1, u3)
   x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UX, kx); x2 = Y(Y_UZ, kx); }, z, ex, q, scale);
-  {
-    T s = T(0);
+  put(0, sq2);
 #pragma unroll
-    for (int b = 0; b < 16; ++b) { s += z[b].x * z[b].x + z[b].y * z[b].y; s13[b] = fabs(z[b].x) + fabs(z[b].y); }
-    acc[0].add(s);
-  }
+  for (int b = 0; b < 16; ++b) s13[b] = fabs(z[b].x) + fabs(z[b].y);
   // (u2, phi)
   x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = Y(Y_UY, kx); x2 = Y(Y_PHI, kx); }, z, ex, q, scale);
-  {
-    T s0 = T(0), s1 = T(0), s2 = T(0);
+  put(0, [&](int b) { return z[b].x * z[b].x; });
+  put(20, [&](int b) { return z[b].y * z[b].x; });
+  put(21, [&](int b) { return z[b].y * z[b].y; });
 #pragma unroll
-    for (int b = 0; b < 16; ++b) {
-      s0 += z[b].x * z[b].x; s1 += z[b].y * z[b].x; s2 += z[b].y * z[b].y;
-      um = max_keep_nan(um, s13[b] + fabs(z[b].x));
-    }
-    acc[0].add(s0);
-    acc[20].add(s1);
-    acc[21].add(s2);
-  }
+  for (int b = 0; b < 16; ++b) um = max_keep_nan(um, s13[b] + fabs(z[b].x));
   // (omega1, omega2)
   x2inv<T, N, true, KK>(
       [&](int kx, C& x1, C& x2) { x1 = Y(Y_WX, kx); x2 = csub(Y(Y_DZUX, kx), mul_ik(Y(Y_UZ, kx), T(kx))); }, z, ex, q,
       scale);
-  {
-    T s = T(0);
-#pragma unroll
-    for (int b = 0; b < 16; ++b) s += z[b].x * z[b].x + z[b].y * z[b].y;
-    acc[1].add(s);
-  }
+  put(1, sq2);
   // (omega3, dphi/dx1)
   x2inv<T, N, true, KK>(
       [&](int kx, C& x1, C& x2) {
@@ -542,13 +541,8 @@ __device__ __forceinline__ bool x2_stats_row(const YF& Y, const HA& after_a, con
         x2 = mul_ik(Y(Y_PHI, kx), T(kx));
       },
       z, ex, q, scale);
-  {
-    T s = T(0);
-#pragma unroll
-    for (int b = 0; b < 16; ++b) s += z[b].x * z[b].x;
-    acc[1].add(s);
-    mom3(11, im);
-  }
+  put(1, [&](int b) { return z[b].x * z[b].x; });
+  mom3(11, im);
   // (du1/dx1, du2/dx2)
   x2inv<T, N, true, KK>([&](int kx, C& x1, C& x2) { x1 = mul_ik(Y(Y_UX, kx), T(kx)); x2 = Y(Y_DYUY, kx); }, z, ex, q,
                         scale);
