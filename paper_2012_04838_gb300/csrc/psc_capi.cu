@@ -15,6 +15,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "psc.h"
+#include "psc_batch_plan.h"
 #include "psc_kernels.cuh"
 
 // ---------------------------------------------------------------- dispatch
@@ -1139,59 +1140,25 @@ psc_status psc_batch_create(psc_sim* const* sims, int32_t n, void* stream, psc_b
     launch0[i] = sims[i]->launches;
     sims[i]->pdl = 0;
   }
-  // The members' steps as a graph: the largest first, each forked off as soon as
-  // the workspaces of the members under way leave room for its own within
-  // kBatchBytes (by a model of their run times: grid points and a constant), so
-  // that small boxes fill the chip together while what they stream stays near
-  // the L2 cache's size.  48 x 64^3 + 12 x 96^3 + 3 x 128^3, ms a step: all 63 at
-  // once 4.92; 20 / 60 / 110 / 180 / 240 / 400 / 1000 MB under way 8.92 / 5.84 /
-  // 4.82 / 4.61 / 4.37 / 4.35 / 4.59.
-  constexpr size_t kBatchBytes = (size_t)320 << 20;
-  // The tile variants were measured with a box alone on the chip.  Where the
-  // members keep the chip full instead (their workspaces exceed what is let under
-  // way), the staged 8-column variant is faster in every strided pass than the
-  // measured mixture, whose wider and unstaged tiles pay by filling idle SMs:
-  // us a step, measured mixture -> staged, 48 x 64^3 + 12 x 96^3 + 3 x 128^3
-  // 4357 -> 4249, 24 x 64^3 943 -> 926, 8 x 96^3 1077 -> 1050, 3 x 128^3 1045 ->
-  // 1030; 4 x 64^3, which leave room, 172 -> 175.  All variants give the same bits.
-  size_t total = 0;
-  for (int i = 0; i < n; ++i) total += sims[i]->L.total;
-  const bool full = total > kBatchBytes;
-  std::vector<int> order(n);
-  for (int i = 0; i < n; ++i) order[i] = i;
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return sims[x]->L.total > sims[y]->L.total; });
-  struct Running {
-    double end;
-    int i;
-  };
-  std::vector<Running> run;
-  size_t used = 0;
-  double clock = 0.0;
-  int last = -1;  // the member whose end made room last
+  // the members' steps as a graph: who waits for whom is batch_plan()'s
+  std::vector<PlanMember> sizes(n);
+  for (int i = 0; i < n; ++i) sizes[i] = PlanMember{sims[i]->L.total, sims[i]->d.N};
+  const std::vector<PlanStart> plan = batch_plan(sizes);
   cudaError_t e = cudaStreamBeginCapture(b->st, cudaStreamCaptureModeRelaxed);
   psc_status st = PSC_OK;
   if (e == cudaSuccess) e = cudaEventRecord(b->events[0], b->st);
   for (int k = 0; k < n && e == cudaSuccess && st == PSC_OK; ++k) {
-    const int i = order[k];
+    const int i = plan[k].member;
     psc_sim* m = sims[i];
     if (m->st != b->st) e = cudaStreamWaitEvent(m->st, b->events[0], 0);
-    while (!run.empty() && used + m->L.total > kBatchBytes && e == cudaSuccess) {
-      auto it = std::min_element(run.begin(), run.end(), [](const Running& x, const Running& y) { return x.end < y.end; });
-      clock = std::max(clock, it->end);
-      last = it->i;
-      used -= sims[last]->L.total;
-      run.erase(it);
-      e = cudaStreamWaitEvent(m->st, b->events[last + 1], 0);
-    }
-    if (last >= 0 && e == cudaSuccess) e = cudaStreamWaitEvent(m->st, b->events[last + 1], 0);
+    for (int j : plan[k].after)
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(m->st, b->events[j + 1], 0);
     if (e != cudaSuccess) break;
-    const double N = m->d.N;
-    used += m->L.total;
-    run.push_back(Running{clock + N * N * N + 3.0e5, i});
-    m->share = (int)std::max<size_t>(1, std::min<size_t>(n, kBatchBytes / m->L.total));
+    m->share = plan[k].share;
     int wv[SP_N];
     std::copy(m->wv, m->wv + SP_N, wv);
-    if (full && m->tuned && !m->fp64 && !m->d.sph)
+    // all variants give the same bits
+    if (plan[k].crowd && m->tuned && !m->fp64 && !m->d.sph)
       for (int v = 0; v < m->tb->nvariants; ++v)
         for (int p = 0; p < SP_N; ++p)
           if (m->tb->staged[v] && m->tb->widths[v] == 8 && ((m->tb->vmask[p] >> v) & 1u)) m->wv[p] = v;
