@@ -29,7 +29,6 @@ template <typename T, int N> struct X2Cfg {
   static constexpr int ROW = 17 * G;
   static constexpr int EXCH = 16 * ROW > N ? 16 * ROW : N;
   static constexpr size_t LINE_BYTES = (EXCH * sizeof(C) + 15) / 16 * 16;
-  static constexpr size_t ACC_BYTES = 4 * NQ * sizeof(double);
   // per-role twiddle tables (every row of the CTA uses the same thread roles):
   //   T1[a][tid]  = wN^(a tid)             (inverse step after the first DFT-16)
   //   T3[k1][tid] = wN^(ra (rk0 + G k1))   (forward step before the exchange)
@@ -37,7 +36,7 @@ template <typename T, int N> struct X2Cfg {
   // laid out so the 32 lanes of a warp read consecutive entries (FP32: pairs
   // of consecutive a, k1 or b side by side, see tw_index)
   static constexpr size_t TW_BYTES = (size_t)(2 * 16 * TH + 16 * G) * sizeof(C);
-  static constexpr size_t SMEM = LINE_BYTES * ROWS + ACC_BYTES + TW_BYTES;
+  static constexpr size_t SMEM = LINE_BYTES * ROWS + TW_BYTES;
   static constexpr int K = (N - 1) / 3;
   static_assert(N == 256 || N == 512 || N == 1024, "X2 layout covers N = 256, 512 and 1024");
 };
@@ -586,12 +585,11 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : PSC_X2_MINB) k_xpass
   q.rk0 = bitrev_lane<G>(q.rr);
   q.bar = 1 + lid;
   C* ex = reinterpret_cast<C*>(smraw + (size_t)lid * XC::LINE_BYTES);
-  double* accw = reinterpret_cast<double*>(smraw + XC::LINE_BYTES * ROWS) + wid * NQ;
   const C* __restrict__ yb = static_cast<const C*>(a.yb);
   C* __restrict__ xb = static_cast<C*>(a.xb);
   const C* __restrict__ tw = static_cast<const C*>(a.tw);
   pdl_trigger(a.pdl);
-  x2_twiddles<T, N>(reinterpret_cast<C*>(smraw + XC::LINE_BYTES * ROWS + XC::ACC_BYTES), tw, q);
+  x2_twiddles<T, N>(reinterpret_cast<C*>(smraw + XC::LINE_BYTES * ROWS), tw, q);
   pdl_wait(a.pdl);
   // rows and the stream stride come from the arguments (N*N rows for a pass over the box)
   const long long ys = a.d.ys;
@@ -640,7 +638,6 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : PSC_X2_MINB) k_xpass
       if (lane == 0) a.partials[gw * NQ + i] = v;
     }
   }
-  (void)accw;
 }
 
 // ---------------------------------------------------------------------------
