@@ -196,8 +196,8 @@ psc_status psc_time(psc_sim* s, double* t, int64_t* step, double* dt);
  * psc_batch_create() captures one RK4 step of every member into a single CUDA
  * graph, each member's work on its own stream, forked from and joined back into
  * `stream`; psc_batch_step() replays that graph, so an ensemble step costs one
- * graph launch and small boxes run concurrently (the largest first, as many at a
- * time as fit a budget of workspace bytes).
+ * graph launch and boxes run concurrently (the largest first; of many small ones
+ * as many at a time as fit a budget of workspace bytes).
  * Each member advances exactly as psc_step() would advance it (the step counter
  * and the CFL decision live on the device).  Members need non-NULL streams;
  * members that share a stream become consecutive steps of one branch (correct,

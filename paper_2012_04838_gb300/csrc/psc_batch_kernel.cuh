@@ -263,7 +263,10 @@ constexpr unsigned long long kStallTestWaitNs = 50000000ull;
 
 #ifndef PSCB_MINB
 // CTAs per SM the register budget is sized for (63 boxes, ms a step: 3 / 4 / 5 / 6
-// CTAs 8.24 / 7.44 / 7.86 / 7.93; more of them spill)
+// CTAs 8.24 / 7.44 / 7.86 / 7.93; more of them spill).  The kernel of every size
+// (BIG), us a step with 3 / 4: 256^3 5673 / 5382, 2 x 256^3 8957 / 8469, 192^3 2872 / 2566,
+// 4 x 192^3 6573 / 6076, 256^3 + 24 x 64^3 6951 / 6450, two each of 256 192 128 96 64 13785 / 13100;
+// three 128^3 in it 2344 / 2515
 #define PSCB_MINB 4
 #endif
 template <int STAGE, bool BIG>

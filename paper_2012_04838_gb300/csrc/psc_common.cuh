@@ -97,8 +97,8 @@ template <int N> struct PlanD : Plan<N> {
 // by 1/N^3, which their X passes' inverse twiddle tables carry (a multiplication of
 // every value at the end instead cost the convective 256^3 step 2.4%).  The others
 // leave the fields N^3 times too large and scale each product by 1/N^6: in FP32 that
-// holds while
-// |u| |omega| and |u| |grad phi| stay below 3.4e38 / N^6 (1e22 at 512, 2.9e20 at 1024).
+// holds while |u| |omega| and |u| |grad phi| stay below 3.4e38 / N^6 (1.9e22 at 512,
+// 2.9e20 at 1024).  The row X pass (520) always scales.
 template <typename T, int N> constexpr bool kScaled = sizeof(T) == 4 && N < 512;
 
 // Programmatic dependent launch: a pass is launched while the one before it in

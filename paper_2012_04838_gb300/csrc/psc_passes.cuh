@@ -14,8 +14,9 @@
 //   Y-forward : lines along y, forward DFT, keep |ky| <= K
 //   Z-forward : lines along z, forward DFT, keep |kz| <= K -> compact RHS
 //
-// All transforms are the unnormalised DFTs of Eq. 5; the 1/N^3 of the
-// inverse is applied once, to the physical fields in the X pass.
+// All transforms are the unnormalised DFTs of Eq. 5; the inverse's 1/N^3 is
+// applied in the X pass: to the physical fields in the statistics and in the
+// products of FP32 grids below 512, as 1/N^6 to each product elsewhere (kScaled).
 #pragma once
 
 #include <atomic>
@@ -470,7 +471,8 @@ __host__ __device__ constexpr int slot_band(int N, int s0, int w, int K) {
 // conj(X1[N-p]) + i conj(X2[N-p]) (p >= N-K), 0 elsewhere.  On return
 // z[j][k2] holds scale * IDFT(Z) at position (t + j TPL) + R1 k2, whose real
 // and imaginary parts are the two real fields (SCALE = false: the unscaled
-// IDFT; the caller folds 1/N^3 into its products).  A slot's TPL positions lie
+// IDFT; the caller folds 1/N^3 into its products.  Where kScaled, tw holds the
+// scale already).  A slot's TPL positions lie
 // on adjacent lanes, so which slots are retained, zero or mixed is known when
 // the kernel is compiled: zero slots are neither read nor transformed.
 template <typename T, int N, bool SCALE, int KK = (N - 1) / 3, bool SHIFT = false, class SPEC>

@@ -30,7 +30,8 @@ template <typename T, int N> struct X2Cfg {
   static constexpr int EXCH = 16 * ROW > N ? 16 * ROW : N;
   static constexpr size_t LINE_BYTES = (EXCH * sizeof(C) + 15) / 16 * 16;
   // per-role twiddle tables (every row of the CTA uses the same thread roles):
-  //   T1[a][tid]  = wN^(a tid)             (inverse step after the first DFT-16)
+  //   T1[a][tid]  = wN^(a tid)             (inverse step after the first DFT-16;
+  //                                         times 1/N^3 where kScaled)
   //   T3[k1][tid] = wN^(ra (rk0 + G k1))   (forward step before the exchange)
   //   T2[b][k0]   = wN^(16 b k0)           (between the lane DFT and the DFT-16 over b)
   // laid out so the 32 lanes of a warp read consecutive entries (FP32: pairs
@@ -161,7 +162,8 @@ __device__ __forceinline__ void tw_pair(const typename CT<T>::type* t, int e, in
 // Z[p] = X1[p] + i X2[p] (p <= K, imaginary parts dropped at p = 0),
 // conj(X1[N-p]) + i conj(X2[N-p]) (p >= N-K), 0 elsewhere.  On return
 // z[b] = scale * IDFT(Z) at n = ra + 16 b + 256 rr (SCALE = false: the
-// unscaled IDFT; the caller folds 1/N^3 into its products).
+// unscaled IDFT; the caller folds 1/N^3 into its products.  Where kScaled, T1
+// holds the scale already).
 template <typename T, int N, bool SCALE = true, int KK = (N - 1) / 3, bool SHIFT = false, class SPEC>
 __device__ __forceinline__ void x2inv(const SPEC& spec, typename CT<T>::type (&z)[16],
                                       typename CT<T>::type* ex, const X2Roles<typename CT<T>::type>& q,
